@@ -537,11 +537,9 @@ int vie_rhs(vie_op* op, const vie_incident* inc, int nrhs, void* b, int64_t ld, 
         if (ld < o.n()) fail(VIE_ERR_INVALID_ARG, "ld < n");
         check_vectors("vie_rhs", b, nullptr, 0);
         cudaStream_t s = stream ? (cudaStream_t)stream : o.ctx->stream;
-        DevBuf kh(3 * nrhs * sizeof(double)), pl(6 * nrhs * sizeof(double));
-        VIE_CUDA(cudaMemcpyAsync(kh.p, inc->khat, 3 * nrhs * sizeof(double), cudaMemcpyHostToDevice, s));
-        VIE_CUDA(cudaMemcpyAsync(pl.p, inc->pol, 6 * nrhs * sizeof(double), cudaMemcpyHostToDevice, s));
-        rhs_kernel_launch(o, kh.as<double>(), pl.as<double>(), nrhs, b, ld, s);
-        VIE_CUDA(cudaStreamSynchronize(s));
+        const IncidentDev w = upload_incident(o, inc, nrhs, s);
+        rhs_kernel_launch(o, w.khat, w.pol, nrhs, b, ld, s);
+        VIE_CUDA(cudaStreamSynchronize(s));  // the operator's tables are free for the next call on any stream
     });
 }
 
@@ -581,6 +579,34 @@ int vie_solve_batch(vie_op* const* ops, int count, const vie_incident* inc, cons
     return result;
 }
 
+// nt-point Gauss-Legendre in cos(theta) x nph-point trapezoid in phi: unit
+// directions (3 per point) and weights
+static void sphere_rule(int nt, int nph, std::vector<double>& d, std::vector<double>& wt) {
+    for (int i = 0; i < nt; ++i) {
+        // Newton on the Legendre polynomial P_nt
+        double z = std::cos(M_PI * (i + 0.75) / (nt + 0.5)), w = 0;
+        for (int it = 0; it < 100; ++it) {
+            double p1 = 1, p2 = 0;
+            for (int j = 1; j <= nt; ++j) {
+                const double p3 = p2;
+                p2 = p1;
+                p1 = ((2.0 * j - 1.0) * z * p2 - (j - 1.0) * p3) / j;
+            }
+            const double pp = nt * (z * p1 - p2) / (z * z - 1.0), z1 = z;
+            z = z1 - p1 / pp;
+            w = 2.0 / ((1.0 - z * z) * pp * pp);
+            if (std::fabs(z - z1) < 1e-15) break;
+        }
+        for (int j = 0; j < nph; ++j) {
+            const double st = std::sqrt(1 - z * z), ph = 2 * M_PI * j / nph;
+            d.push_back(st * std::cos(ph));
+            d.push_back(st * std::sin(ph));
+            d.push_back(z);
+            wt.push_back(w * 2 * M_PI / nph);
+        }
+    }
+}
+
 int vie_fields(vie_op* op, const vie_incident* inc, const void* I, int nrhs, const double* dirs, int npts, int mode,
                void* E_out, double* sigma_out) {
     if (!op || !I || nrhs < 1) return VIE_ERR_INVALID_ARG;
@@ -590,98 +616,60 @@ int vie_fields(vie_op* op, const vie_incident* inc, const void* I, int nrhs, con
         if (mode != 0 && mode != 1) fail(VIE_ERR_INVALID_ARG, "vie_fields: mode 0 (far field) or 1 (near field)");
         cudaStream_t s = o.ctx->stream;
         const int64_t n = o.n();
-        DevBuf dI((size_t)n * nrhs * sizeof(double2));
-        VIE_CUDA(cudaMemcpyAsync(dI.p, I, dI.bytes, cudaMemcpyHostToDevice, s));
         if (mode == 1) {
             if (!E_out || !dirs || npts < 1) fail(VIE_ERR_INVALID_ARG, "vie_fields: the near field needs points and E_out");
             for (int64_t i = 0; i < 3 * (int64_t)npts; ++i)
                 if (!std::isfinite(dirs[i])) fail(VIE_ERR_INVALID_ARG, "vie_fields: non-finite point");
-            DevBuf dp((size_t)3 * npts * sizeof(double)), out((size_t)npts * nrhs * 3 * sizeof(double2));
-            VIE_CUDA(cudaMemcpyAsync(dp.p, dirs, dp.bytes, cudaMemcpyHostToDevice, s));
-            near_field_launch(o, dI.p, nrhs, dp.as<double>(), npts, out.p, s);
-            VIE_CUDA(cudaMemcpyAsync(E_out, out.p, out.bytes, cudaMemcpyDeviceToHost, s));
-            VIE_CUDA(cudaStreamSynchronize(s));
-            if (sigma_out) fail(VIE_ERR_INVALID_ARG, "vie_fields: cross sections come with mode 0");
-            return;
         }
-        auto far = [&](const std::vector<double>& d, std::vector<cd>& F) {
-            int np_ = (int)(d.size() / 3);
-            DevBuf dd(d.size() * sizeof(double)), out((size_t)np_ * nrhs * 3 * sizeof(double2));
-            VIE_CUDA(cudaMemcpyAsync(dd.p, d.data(), dd.bytes, cudaMemcpyHostToDevice, s));
-            far_field_launch(o, dI.p, nrhs, dd.as<double>(), np_, out.p, s);
-            std::vector<cd> N((size_t)np_ * nrhs * 3);
-            VIE_CUDA(cudaMemcpyAsync(N.data(), out.p, out.bytes, cudaMemcpyDeviceToHost, s));
-            VIE_CUDA(cudaStreamSynchronize(s));
-            // F = -j k / (4 pi) (N - rhat (rhat . N))
-            F.resize(N.size());
-            for (int c = 0; c < nrhs; ++c)
-                for (int p = 0; p < np_; ++p) {
-                    const double* r = &d[3 * p];
-                    cd* v = &N[((size_t)c * np_ + p) * 3];
-                    cd dot = r[0] * v[0] + r[1] * v[1] + r[2] * v[2];
-                    for (int e = 0; e < 3; ++e)
-                        F[((size_t)c * np_ + p) * 3 + e] = cd(0, -o.k / (4 * M_PI)) * (v[e] - r[e] * dot);
-                }
+        // the call ends synchronised, so the operator's field workspaces are free
+        // again; the large ones are given back
+        struct Trim {
+            Op& o;
+            ~Trim() {
+                cudaStreamSynchronize(o.ctx->stream);
+                for (DevBuf* b : {&o.d_fI, &o.d_fdirs, &o.d_fout, &o.d_fpart})
+                    if (b->bytes > Op::kFieldsKeep) b->release();
+            }
+        } trim{o};
+        auto grow = [](DevBuf& b, size_t bytes) {
+            if (b.bytes < bytes) b.alloc(bytes);
         };
+        grow(o.d_fI, (size_t)n * nrhs * sizeof(double2));
+        VIE_CUDA(cudaMemcpyAsync(o.d_fI.p, I, (size_t)n * nrhs * sizeof(double2), cudaMemcpyHostToDevice, s));
         if (E_out && dirs && npts > 0) {
-            std::vector<double> d(dirs, dirs + 3 * npts);
-            std::vector<cd> F;
-            far(d, F);
-            std::memcpy(E_out, F.data(), F.size() * sizeof(cd));
+            const size_t out_b = (size_t)npts * nrhs * 3 * sizeof(double2);
+            grow(o.d_fdirs, (size_t)3 * npts * sizeof(double));
+            grow(o.d_fout, out_b);
+            VIE_CUDA(cudaMemcpyAsync(o.d_fdirs.p, dirs, (size_t)3 * npts * sizeof(double), cudaMemcpyHostToDevice, s));
+            if (mode == 1) near_field_launch(o, o.d_fI.p, nrhs, o.d_fdirs.as<double>(), npts, o.d_fout.p, s);
+            else far_field_launch(o, o.d_fI.p, nrhs, o.d_fdirs.as<double>(), npts, o.d_fout.p, s);
+            VIE_CUDA(cudaMemcpyAsync(E_out, o.d_fout.p, out_b, cudaMemcpyDeviceToHost, s));
+            VIE_CUDA(cudaStreamSynchronize(s));
         }
         if (sigma_out) {
+            if (mode == 1) fail(VIE_ERR_INVALID_ARG, "vie_fields: cross sections come with mode 0");
             if (!inc) fail(VIE_ERR_INVALID_ARG, "cross sections need the incident field");
-            // 24-point Gauss-Legendre in cos(theta) x 48-point trapezoid in phi
-            const int nt = 24, nph = 48;
-            std::vector<double> x(nt), w(nt);
-            for (int i = 0; i < nt; ++i) {  // Newton on P_n
-                double z = std::cos(M_PI * (i + 0.75) / (nt + 0.5));
-                for (int it = 0; it < 100; ++it) {
-                    double p1 = 1, p2 = 0;
-                    for (int j = 1; j <= nt; ++j) {
-                        double p3 = p2;
-                        p2 = p1;
-                        p1 = ((2.0 * j - 1.0) * z * p2 - (j - 1.0) * p3) / j;
-                    }
-                    double pp = nt * (z * p1 - p2) / (z * z - 1.0);
-                    double z1 = z;
-                    z = z1 - p1 / pp;
-                    if (std::fabs(z - z1) < 1e-15) {
-                        w[i] = 2.0 / ((1.0 - z * z) * pp * pp);
-                        break;
-                    }
-                    w[i] = 2.0 / ((1.0 - z * z) * pp * pp);
-                }
-                x[i] = z;
+            const int nt = 24, nph = 48, nd = nt * nph;
+            if (!o.d_sphere.p) {  // directions, then weights, of the quadrature sphere
+                std::vector<double> d, wt;
+                sphere_rule(nt, nph, d, wt);
+                d.insert(d.end(), wt.begin(), wt.end());
+                upload(o.d_sphere, d);
             }
-            std::vector<double> d, wt;
-            for (int i = 0; i < nt; ++i)
-                for (int j = 0; j < nph; ++j) {
-                    double st_ = std::sqrt(1 - x[i] * x[i]), ph = 2 * M_PI * j / nph;
-                    d.push_back(st_ * std::cos(ph));
-                    d.push_back(st_ * std::sin(ph));
-                    d.push_back(x[i]);
-                    wt.push_back(w[i] * 2 * M_PI / nph);
-                }
-            std::vector<cd> F;
-            far(d, F);
-            // extinction Re(I^H v0), v0 = b / (j k)
-            DevBuf b((size_t)n * nrhs * sizeof(double2)), kh(3 * nrhs * sizeof(double)), pl(6 * nrhs * sizeof(double));
-            VIE_CUDA(cudaMemcpyAsync(kh.p, inc->khat, kh.bytes, cudaMemcpyHostToDevice, s));
-            VIE_CUDA(cudaMemcpyAsync(pl.p, inc->pol, pl.bytes, cudaMemcpyHostToDevice, s));
-            rhs_kernel_launch(o, kh.as<double>(), pl.as<double>(), nrhs, b.p, n, s);
-            std::vector<cd> hb((size_t)n * nrhs);
-            VIE_CUDA(cudaMemcpyAsync(hb.data(), b.p, b.bytes, cudaMemcpyDeviceToHost, s));
+            const double* sph = o.d_sphere.as<double>();
+            grow(o.d_fout, (size_t)nd * nrhs * 3 * sizeof(double2) + 2 * nrhs * sizeof(double));
+            double2* F = o.d_fout.as<double2>();
+            double* res = reinterpret_cast<double*>(F + (size_t)nd * nrhs * 3);
+            const IncidentDev w = upload_incident(o, inc, nrhs, s);
+            far_field_launch(o, o.d_fI.p, nrhs, sph, nd, F, s);
+            sphere_sum_launch(F, sph + 3 * nd, nd, nrhs, res + nrhs, s);
+            extinction_launch(o, o.d_fI.p, w.khat, w.pol, nrhs, res, s);
+            std::vector<double> h(2 * nrhs);
+            VIE_CUDA(cudaMemcpyAsync(h.data(), res, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
             VIE_CUDA(cudaStreamSynchronize(s));
-            const cd* hI = static_cast<const cd*>(I);
             for (int c = 0; c < nrhs; ++c) {
-                cd acc = 0;
-                for (int64_t i = 0; i < n; ++i) acc += std::conj(hI[i + c * n]) * hb[i + c * n] / cd(0, o.k);
-                double sca = 0;
-                for (size_t p = 0; p < wt.size(); ++p)
-                    for (int e = 0; e < 3; ++e) sca += wt[p] * std::norm(F[((size_t)c * wt.size() + p) * 3 + e]);
-                sigma_out[2 * c] = acc.real();
-                sigma_out[2 * c + 1] = sca;
+                sigma_out[2 * c] = h[c];
+                sigma_out[2 * c + 1] = h[nrhs + c];
             }
         }
     });

@@ -190,12 +190,8 @@ int solve_batch(const std::vector<Op*>& ops, const vie_incident* incs, const int
     DevBuf b((size_t)n * K * sizeof(double2)), X((size_t)n * K * sizeof(double2));
     VIE_CUDA(cudaMemsetAsync(b.p, 0, b.bytes, s));
     for (int p = 0; p < B; ++p) {
-        DevBuf kh(3 * nrhs[p] * sizeof(double)), pl(6 * nrhs[p] * sizeof(double));
-        VIE_CUDA(cudaMemcpyAsync(kh.p, incs[p].khat, 3 * nrhs[p] * sizeof(double), cudaMemcpyHostToDevice, s));
-        VIE_CUDA(cudaMemcpyAsync(pl.p, incs[p].pol, 6 * nrhs[p] * sizeof(double), cudaMemcpyHostToDevice, s));
-        rhs_kernel_launch(*ops[p], kh.as<double>(), pl.as<double>(), nrhs[p],
-                          b.as<double2>() + (int64_t)cbeg[p] * n + lo[p], n, s);
-        VIE_CUDA(cudaStreamSynchronize(s));  // kh, pl go out of scope
+        const IncidentDev w = upload_incident(*ops[p], &incs[p], nrhs[p], s);
+        rhs_kernel_launch(*ops[p], w.khat, w.pol, nrhs[p], b.as<double2>() + (int64_t)cbeg[p] * n + lo[p], n, s);
     }
     const GmresOutcome r = run_gmres(*U, lay, b.as<double2>(), X.as<double2>(), *o, K);
     const double tol = o->tol > 0 ? o->tol : 1e-6;

@@ -223,6 +223,12 @@ struct Op {
     // scratch
     DevBuf d_t, d_F;
     DevBuf d_xs;  // float64 vectors split into float32 head + tail (double-float apply)
+    // plane waves and fields: incident directions and polarisations, plane-wave
+    // tables (at most 32 MB, or one direction's), partial sums, currents, results,
+    // and the quadrature sphere of the cross sections.  What a vie_fields call
+    // leaves above kFieldsKeep is given back when it returns.
+    DevBuf d_inc, d_pw, d_fpart, d_fI, d_fdirs, d_fout, d_sphere;
+    static constexpr size_t kFieldsKeep = (size_t)64 << 20;
     size_t t_cap = 0, F_cap = 0;
     double t_assemble = 0, t_compress = 0;
     // compression method of the stored factors (0: range finder, 1: cross
@@ -308,13 +314,20 @@ void assemble_pairs_f32_from_f64(Op& op, const PairJob* d_jobs, int n_jobs, void
                                  cudaStream_t s, double* norm_out = nullptr);
 void dense_apply_c64(Op& op, const float2* x, float2* y, cudaStream_t s);
 void dense_apply_c128(Op& op, const double2* x, double2* y, cudaStream_t s);
+// fields.cu (float64; all work on `s`, workspaces of the operator)
+// incident waves into op.d_inc: directions (3 per wave), then polarisations (6 per wave)
+struct IncidentDev {
+    const double *khat, *pol;
+};
+IncidentDev upload_incident(Op& op, const vie_incident* inc, int nrhs, cudaStream_t s);
 void rhs_kernel_launch(Op& op, const double* d_khat, const double* d_pol, int nrhs, void* b, int64_t ld,
                        cudaStream_t s);
 void near_field_launch(Op& op, const void* d_I, int nrhs, const double* d_pts, int npts, void* d_out, cudaStream_t s);
 void far_field_launch(Op& op, const void* d_I, int nrhs, const double* d_dirs, int npts, void* d_out,
                       cudaStream_t s);
-void v0_dot_launch(Op& op, const void* d_I, const double* d_khat, const double* d_pol, int nrhs,
-                   double* d_out, cudaStream_t s);
+void extinction_launch(Op& op, const void* d_I, const double* d_khat, const double* d_pol, int nrhs, double* d_ext,
+                       cudaStream_t s);
+void sphere_sum_launch(const void* d_F, const double* d_wt, int npts, int nrhs, double* d_sca, cudaStream_t s);
 
 // linalg.cu
 void invert_self_blocks(Op& op);   // d_inv64 from d_zself64 (Gauss-Jordan, partial pivoting)

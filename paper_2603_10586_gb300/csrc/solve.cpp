@@ -556,11 +556,9 @@ int solve(Op& op, const vie_incident* inc, int nrhs, const vie_solve_opts* o, vo
     cudaStream_t s = op.ctx->stream;
     const int64_t n = op.n();
     double t0 = now_s();
-    DevBuf kh(3 * nrhs * sizeof(double)), pl(6 * nrhs * sizeof(double));
-    VIE_CUDA(cudaMemcpyAsync(kh.p, inc->khat, 3 * nrhs * sizeof(double), cudaMemcpyHostToDevice, s));
-    VIE_CUDA(cudaMemcpyAsync(pl.p, inc->pol, 6 * nrhs * sizeof(double), cudaMemcpyHostToDevice, s));
     DevBuf b((size_t)n * nrhs * sizeof(double2));
-    rhs_kernel_launch(op, kh.as<double>(), pl.as<double>(), nrhs, b.p, n, s);
+    const IncidentDev w = upload_incident(op, inc, nrhs, s);
+    rhs_kernel_launch(op, w.khat, w.pol, nrhs, b.p, n, s);
     DevBuf xdev;
     double2* X;
     if (o->out_on_device) X = static_cast<double2*>(I_out);
