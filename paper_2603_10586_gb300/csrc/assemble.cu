@@ -167,22 +167,40 @@ __device__ int surf_rect(const DevMesh& m, int s, double h, double lo[3], double
 
 // The voxel/voxel integrals of one atom depend only on the relative offset of
 // the two voxels (uniform voxels, local coordinates), so they are computed
-// once per offset o = ijk_B - ijk_A in [-(nv-1), nv-1]^3, one warp each: the
-// lanes split the outer points of both rules and all-reduce the sums; a
-// second kernel copies them to every voxel pair.  Rules: 3-point Gauss per
-// axis on both voxels (full g apart, smooth remainder when touching); for
-// touching voxels the static part with a 6-point outer rule and the closed-form
-// box potentials inside.
-__device__ __forceinline__ double warp_allsum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// once per offset o = ijk_B - ijk_A in [-(nv-1), nv-1]^3, one CTA each: the
+// threads split the 729 point pairs of the 3-point rules (full g apart, smooth
+// remainder when touching) and, for touching voxels, the 216 outer points of
+// the static part (6-point rule, closed-form box potentials inside); a second
+// kernel copies the sums to every voxel pair.  A closed form is a serial chain
+// of ~50 float64 logarithms and arctangents per outer point, so the time is the
+// longest chain of one thread: one outer point each (256 threads) instead of
+// seven (a warp per offset) takes 0.58 instead of 1.98 ms at 3 voxels per edge.
+constexpr int kSelfThr = 256;
+constexpr int kVvSums = 13;  // U, then W[d][sa][sb]
+
+// sums of K values over the CTA, valid in every thread (fixed order)
+template <int K>
+__device__ __forceinline__ void cta_allsum(double (&v)[K], double (*sh)[K]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
+    __syncthreads();  // sh of an earlier sum has been read
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < K; ++i) sh[warp][i] = v[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        v[i] = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v[i] += sh[w][i];
+    }
 }
 
-__global__ void __launch_bounds__(128) self_vv_offset_kernel(int nv, double h, double k, double2* otab) {
-    const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kSelfThr) self_vv_offset_kernel(int nv, double h, double k, double2* otab) {
+    const int off = blockIdx.x, tid = threadIdx.x;
     const int w1 = 2 * nv - 1, noff = w1 * w1 * w1;
-    if (warp >= noff) return;  // whole warps
-    const int o[3] = {warp / (w1 * w1) - (nv - 1), (warp / w1) % w1 - (nv - 1), warp % w1 - (nv - 1)};
+    const int o[3] = {off / (w1 * w1) - (nv - 1), (off / w1) % w1 - (nv - 1), off % w1 - (nv - 1)};
     double loA[3], loB[3], hiB[3];
     bool touch = true;
     for (int d = 0; d < 3; ++d) {
@@ -193,85 +211,69 @@ __global__ void __launch_bounds__(128) self_vv_offset_kernel(int nv, double h, d
         touch &= abs(o[d]) <= 1;
     }
     const double two_over_lambda = k / kPi;
-    double2 G[3][3][3];
-    for (int d = 0; d < 3; ++d)
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) G[d][a][b] = make_double2(0, 0);
-    if (lane < 27) {
-        const int pa = lane;
-        const int ax = pa / 9, ay = (pa / 3) % 3, az = pa % 3;
-        const double ra[3] = {loA[0] + h * c_gl3_x[ax], loA[1] + h * c_gl3_x[ay], loA[2] + h * c_gl3_x[az]};
-        const double wa = c_gl3_w[ax] * c_gl3_w[ay] * c_gl3_w[az];
-        for (int pb = 0; pb < 27; ++pb) {
-            const int bx = pb / 9, by = (pb / 3) % 3, bz = pb % 3;
-            const double dx = ra[0] - (loB[0] + h * c_gl3_x[bx]);
-            const double dy = ra[1] - (loB[1] + h * c_gl3_x[by]);
-            const double dz = ra[2] - (loB[2] + h * c_gl3_x[bz]);
-            const double R = sqrt(dx * dx + dy * dy + dz * dz);
-            double2 g = touch ? green4pi_smooth(R, k) : green4pi<double>(R, two_over_lambda);
-            g = (wa * c_gl3_w[bx] * c_gl3_w[by] * c_gl3_w[bz]) * g;
-            G[0][ax][bx] += g;
-            G[1][ay][by] += g;
-            G[2][az][bz] += g;
+    __shared__ double sh[kSelfThr / 32][2 * kVvSums];
+    double acc[2 * kVvSums];  // (re, im) of U and of W[d][sa][sb]
+#pragma unroll
+    for (int i = 0; i < 2 * kVvSums; ++i) acc[i] = 0.0;
+    for (int p = tid; p < 729; p += kSelfThr) {
+        const int pa = p / 27, pb = p % 27;
+        const int ia[3] = {pa / 9, (pa / 3) % 3, pa % 3}, ib[3] = {pb / 9, (pb / 3) % 3, pb % 3};
+        double r2 = 0.0, w = 1.0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double t = (loA[d] + h * c_gl3_x[ia[d]]) - (loB[d] + h * c_gl3_x[ib[d]]);
+            r2 += t * t;
+            w *= c_gl3_w[ia[d]] * c_gl3_w[ib[d]];
+        }
+        const double R = sqrt(r2);
+        double2 g = touch ? green4pi_smooth(R, k) : green4pi<double>(R, two_over_lambda);
+        g = w * g;
+        acc[0] += g.x;
+        acc[1] += g.y;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double xa = c_gl3_x[ia[d]], xb = c_gl3_x[ib[d]];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const double pr = ((q & 2) ? 1.0 - xa : xa) * ((q & 1) ? 1.0 - xb : xb);
+                acc[2 * (1 + 4 * d + q)] += pr * g.x;
+                acc[2 * (1 + 4 * d + q) + 1] += pr * g.y;
+            }
         }
     }
-    for (int d = 0; d < 3; ++d)
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) {
-                G[d][a][b].x = warp_allsum(G[d][a][b].x);
-                G[d][a][b].y = warp_allsum(G[d][a][b].y);
-            }
+    cta_allsum<2 * kVvSums>(acc, sh);
     const double scale = h * h * h * h * h * h * kInv4Pi;
-    double2 U = make_double2(0, 0);
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) U += G[0][a][b];
-    U = scale * U;
-    double2 W[3][2][2];
-    for (int d = 0; d < 3; ++d)
-        for (int sa = 0; sa < 2; ++sa)
-            for (int sb = 0; sb < 2; ++sb) {
-                double2 acc = make_double2(0, 0);
-                for (int a = 0; a < 3; ++a)
-                    for (int b = 0; b < 3; ++b) {
-                        const double pa = sa ? 1.0 - c_gl3_x[a] : c_gl3_x[a];
-                        const double pb = sb ? 1.0 - c_gl3_x[b] : c_gl3_x[b];
-                        acc += (pa * pb) * G[d][a][b];
-                    }
-                W[d][sa][sb] = scale * acc;
-            }
-    if (touch) {
-        // static part: outer 6-point rule on A split over the lanes, closed-form inner over B
+#pragma unroll
+    for (int i = 0; i < 2 * kVvSums; ++i) acc[i] *= scale;
+    if (touch) {  // (uniform over the CTA)
+        // static part: outer 6-point rule on A, closed-form inner over B
         const double h3 = h * h * h;
-        double us = 0.0, ws[3][2][2];
-        for (int d = 0; d < 3; ++d)
-            for (int sa = 0; sa < 2; ++sa)
-                for (int sb = 0; sb < 2; ++sb) ws[d][sa][sb] = 0.0;
-        for (int p = lane; p < 216; p += 32) {
+        double st[kVvSums];
+#pragma unroll
+        for (int i = 0; i < kVvSums; ++i) st[i] = 0.0;
+        for (int p = tid; p < 216; p += kSelfThr) {
             const int ix = p / 36, iy = (p / 6) % 6, iz = p % 6;
             const double xi[3] = {c_gl6_x[ix], c_gl6_x[iy], c_gl6_x[iz]};
             const double r[3] = {loA[0] + h * xi[0], loA[1] + h * xi[1], loA[2] + h * xi[2]};
             const double wp = h3 * c_gl6_w[ix] * c_gl6_w[iy] * c_gl6_w[iz] * kInv4Pi;
             const double phi = box_pot(r, loB, hiB);
-            us += wp * phi;
+            st[0] += wp * phi;
+#pragma unroll
             for (int d = 0; d < 3; ++d) {
                 const double lin = box_lin_pot(r, loB, hiB, d, phi);
                 const double inner[2] = {lin, phi - lin};
                 const double prof[2] = {xi[d], 1.0 - xi[d]};
-                for (int sa = 0; sa < 2; ++sa)
-                    for (int sb = 0; sb < 2; ++sb) ws[d][sa][sb] += wp * prof[sa] * inner[sb];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) st[1 + 4 * d + q] += wp * prof[q >> 1] * inner[q & 1];
             }
         }
-        U.x += warp_allsum(us);
-        for (int d = 0; d < 3; ++d)
-            for (int sa = 0; sa < 2; ++sa)
-                for (int sb = 0; sb < 2; ++sb) W[d][sa][sb].x += warp_allsum(ws[d][sa][sb]);
+        cta_allsum<kVvSums>(st, reinterpret_cast<double(*)[kVvSums]>(sh));
+#pragma unroll
+        for (int i = 0; i < kVvSums; ++i) acc[2 * i] += st[i];
     }
-    if (lane == 0) {
-        otab[warp] = U;
-        for (int d = 0; d < 3; ++d)
-            for (int sa = 0; sa < 2; ++sa)
-                for (int sb = 0; sb < 2; ++sb) otab[(size_t)(1 + 4 * d + 2 * sa + sb) * noff + warp] = W[d][sa][sb];
-    }
+    if (tid == 0)
+#pragma unroll
+        for (int i = 0; i < kVvSums; ++i) otab[(size_t)i * noff + off] = make_double2(acc[2 * i], acc[2 * i + 1]);
 }
 
 __global__ void self_vv_expand_kernel(DevMesh m, const double2* __restrict__ otab, double2* __restrict__ tab) {
@@ -285,14 +287,24 @@ __global__ void self_vv_expand_kernel(DevMesh m, const double2* __restrict__ ota
     for (int q = 0; q < 13; ++q) tab[(size_t)q * nv2 + tt] = otab[(size_t)q * noff + idx];
 }
 
+__device__ __forceinline__ double warp_allsum(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // uniform voxel/sheet combinations of one atom with itself
 // mode 0: VS (voxel A, sheet s), 1: SV (sheet s, voxel B), 2: SS
-__global__ void self_surf_kernel(DevMesh m, double h, double k, double2* tab) {
+// One warp per pair: its lanes split the point pairs and, for touching
+// elements, the outer points of the closed forms.  (A thread per pair walked
+// up to 216 closed forms one after another, and the few touching pairs set the
+// time: 8.1 ms at 3 voxels per edge, now 0.59 ms.)
+__global__ void __launch_bounds__(128) self_surf_kernel(DevMesh m, double h, double k, double2* tab) {
     int mode = blockIdx.y;
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     int nA = mode == 2 ? m.nsurf : (mode == 0 ? m.nvox : m.nsurf);
     int nB = mode == 2 ? m.nsurf : (mode == 0 ? m.nsurf : m.nvox);
-    if (t >= nA * nB) return;
+    if (t >= nA * nB) return;  // whole warps
     int ia = t / nB, ib = t % nB;
     const double two_over_lambda = k / kPi;
     // element descriptions
@@ -342,23 +354,20 @@ __global__ void self_surf_kernel(DevMesh m, double h, double k, double2* tab) {
         }
     };
     double2 acc = make_double2(0, 0);
-    for (int p = 0; p < npts(axA); ++p) {
-        double ra[3], wa;
-        point(axA, loA, p, ra, wa);
-        for (int q = 0; q < npts(axB); ++q) {
-            double rb[3], wb;
-            point(axB, loB, q, rb, wb);
-            double dx = ra[0] - rb[0], dy = ra[1] - rb[1], dz = ra[2] - rb[2];
-            double R = sqrt(dx * dx + dy * dy + dz * dz);
-            double2 g = touch ? green4pi_smooth(R, k) : green4pi<double>(R, two_over_lambda);
-            acc += (wa * wb) * g;
-        }
+    for (int e = lane; e < npts(axA) * npts(axB); e += 32) {
+        double ra[3], wa, rb[3], wb;
+        point(axA, loA, e / npts(axB), ra, wa);
+        point(axB, loB, e % npts(axB), rb, wb);
+        double dx = ra[0] - rb[0], dy = ra[1] - rb[1], dz = ra[2] - rb[2];
+        double R = sqrt(dx * dx + dy * dy + dz * dz);
+        double2 g = touch ? green4pi_smooth(R, k) : green4pi<double>(R, two_over_lambda);
+        acc += (wa * wb) * g;
     }
     acc = kInv4Pi * acc;
     if (touch) {
         // static part: outer 6-point rule on the test element, closed-form inner
         int nq = axA < 0 ? 216 : 36;
-        for (int p = 0; p < nq; ++p) {
+        for (int p = lane; p < nq; p += 32) {
             double r[3], wp;
             if (axA < 0) {
                 int i0 = p / 36, i1 = (p / 6) % 6, i2 = p % 6;
@@ -378,6 +387,9 @@ __global__ void self_surf_kernel(DevMesh m, double h, double k, double2* tab) {
             acc.x += wp * inner * kInv4Pi;
         }
     }
+    acc.x = warp_allsum(acc.x);
+    acc.y = warp_allsum(acc.y);
+    if (lane != 0) return;
     size_t nv2 = (size_t)m.nvox * m.nvox;
     size_t base = 13 * nv2;
     if (mode == 0) tab[base + (size_t)ib * m.nvox + ia] = acc;
@@ -703,12 +715,12 @@ void assemble_self_blocks(Op& op) {
         double h = op.h[t];
         int nv2 = m.nvox * m.nvox;
         const int w1 = 2 * m.nv - 1, noff = w1 * w1 * w1;
-        self_vv_offset_kernel<<<(noff * 32 + 127) / 128, 128, 0, s>>>(m.nv, h, op.k, otab.as<double2>());
+        self_vv_offset_kernel<<<noff, kSelfThr, 0, s>>>(m.nv, h, op.k, otab.as<double2>());
         VIE_CHECK_LAUNCH();
         self_vv_expand_kernel<<<(nv2 + 255) / 256, 256, 0, s>>>(m, otab.as<double2>(), tab.as<double2>());
         VIE_CHECK_LAUNCH();
         int ns = std::max(m.nvox, m.nsurf) * m.nsurf;
-        self_surf_kernel<<<dim3((ns + 63) / 64, 3), 64, 0, s>>>(m, h, op.k, tab.as<double2>());
+        self_surf_kernel<<<dim3((ns + 3) / 4, 3), 128, 0, s>>>(m, h, op.k, tab.as<double2>());
         VIE_CHECK_LAUNCH();
         // an atom of this type (entries only need its type); a type without
         // atoms gets an identity block so that its inverse stays defined
