@@ -72,8 +72,10 @@ enum vie_precision {
 /* Implementations of the far part of a complex float32 apply (the paper's
  * method fixes what is computed, not how; these are the kernel variants the
  * autotuner chooses between).  The SIMT variants read every factor element
- * once per group of 1, 2, 4 or 8 right-hand sides; the tensor-core variants
- * compute in split bf16 (admissible for VIE_BF16X3 only). */
+ * once per group of 1, or of at least 2, 4 or 8 right-hand sides (when translated
+ * copies or right-hand sides give a factor three or more columns, all of them run
+ * the register tiles, which take up to 64 columns of a factor together); the
+ * tensor-core variants compute in split bf16 (admissible for VIE_BF16X3 only). */
 enum vie_variant {
     VIE_VAR_AUTO = 0,
     VIE_VAR_SIMT_R1 = 1,
@@ -87,7 +89,7 @@ enum vie_variant {
                                           ~1.1x the factor memory; runs as 6 when that is not free) */
     VIE_VAR_SIMT_SHARED = 8 /* complex float32, one right-hand side at a time: far blocks that share
                                their factors (translated copies) are applied together, each factor
-                               element read once per group of up to 4 copies; partial products are
+                               element read once per group of up to 64 copies; partial products are
                                summed per target atom in a fixed order (default for one right-hand
                                side when the operator has translated copies) */,
     VIE_VAR_TCGEN05_WS_BF16X3 = 9 /* the planes of 7 in a warp-specialised persistent kernel (one CTA

@@ -181,15 +181,17 @@ struct Op {
     int n_p1_items = 0, n_p2_items = 0, n_cta = 0;
     DevBuf d_t1_items, d_t1_cta, d_t2_items, d_t2_cta;  // warp-MMA tensor path (64-row items)
     int n_t1_items = 0, n_t2_items = 0, n_cta_tc = 0;
-    // shared-factor path: blocks with the same factor storage (translated
-    // copies) form a class; members of a class are listed together in
-    // d_cmem and each item covers up to kShareGroup of them.  Phase 2 writes one
-    // partial product per (block, target slot) at d_poff[block] + slot np.
-    DevBuf d_cmem, d_c1_items, d_c1_cta, d_c2_items, d_c2_cta, d_poff, d_part;
-    static constexpr int kShareGroup = 4;  // members per item (register tile of the kernels)
-    int n_c1_items = 0, n_c2_items = 0, n_cta_c = 0;
-    int64_t part_total = 0;             // complex entries of the partial products
-    double share_mean = 1.0;            // far blocks per factor class (rank > 0)
+    // register-tile path (apply_tile.cu): blocks with the same factor storage
+    // (translated copies) form a class, listed in d_cmem in groups of up to
+    // kTileMembers; phase 1 writes t at d_ctoff[block] (one part per tile_seg
+    // columns of R), phase 2 one partial product per (block, target slot) at
+    // d_poff[block] + slot np
+    DevBuf d_cmem, d_c1_items, d_c2_items, d_cseg, d_ctoff, d_poff, d_ct, d_part;
+    static constexpr size_t kTilePass = (size_t)256 << 20;  // partial products of one pass (or one column's)
+    int n_c1_items = 0, n_c2_items = 0, tile_seg = 512;
+    int n_cseg = 0, tile_group = 1;  // blocks with several segments, members of the largest group
+    int64_t ct_total = 0, part_total = 0;  // entries of t and of the partial products per right-hand side
+    double share_mean = 1.0;               // far blocks per factor class (rank > 0)
     // tcgen05 tensor path (built on first use): phase 1 stacks the R rows of
     // all blocks with the same source atoms (one gathered x for up to 128
     // rows), phase 2 walks one virtual K axis over all blocks of an atom
@@ -273,6 +275,14 @@ struct AllocScope {
     explicit AllocScope(Ctx* c);
     ~AllocScope();
 };
+
+// one item of the register-tile apply: the members cmem[first .. first + nm) of
+// a class, rows [row0, row0 + rows) of R (phase 1, columns [k0, k1), segment seg)
+// or of Q (phase 2)
+struct FarTile {
+    int first, nm, row0, rows, k0, k1, seg, pad;
+};
+constexpr int kTileMembers = 64;  // members per item: a full group fills 64-column tiles whatever the right-hand-side count
 
 // device-side block description used by the apply kernels
 struct FarBlockDev {
@@ -370,10 +380,15 @@ size_t umma_pack_bytes(const Op& op);
 void apply_far_umma_packed(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
 void apply_far_umma_ws(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
 void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
-// complex float32 far apply reading each shared factor once per group of up to
-// Op::kShareGroup translated copies (one right-hand side at a time)
-void apply_far_shared(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
-void shared_reserve(Op& op);
+// apply_tile.cu: far apply by register tiles over classes of blocks that share
+// their factors.  tile_reserve: its scratch for nrhs columns of `elem`-byte
+// vector elements; false when the memory is not there (or would have to be allocated
+// while `s` is capturing), and the per-block kernels run instead.
+bool tile_pays(const Op& op, int nrhs);
+bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s);
+template <class TF, class TX, class TO>
+void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nrhs, cudaStream_t s, int first = 0,
+                    int count = -1);  // columns [first, first + count) of the call (-1: all)
 // far part with c64 factors and c128 vectors in double-float arithmetic
 void apply_far_df(Op& op, const double2* x, int64_t ldx, double2* F, int64_t ldf, int nrhs, cudaStream_t s);
 // apply_tc.cu: several right-hand sides on the tensor cores (BF16x3)

@@ -420,62 +420,78 @@ void build_apply_lists(Op& op) {
     upload(op.d_p2_ent, flat.empty() ? std::vector<int2>{make_int2(0, 0)} : flat);
     op.umma_ready = false;
 
-    // shared-factor path: classes of blocks with the same factor storage, in
-    // groups of up to Op::kShareGroup members; phase 1 items of 32 rows of R,
-    // phase 2 items of one target slot and 128 rows of it
+    // register-tile path: classes of blocks with the same factor storage, in
+    // groups of up to kTileMembers members; phase 1 items of up to 64 rows and
+    // tile_seg columns of R, phase 2 items of up to 256 rows of Q.  Rows are cut
+    // into equal pieces (96 = 48 + 48), in storage order: the coarse levels'
+    // long items come first.
     {
         std::map<std::pair<long long, int>, std::vector<int>> cls;
-        std::vector<long long> poff(std::max(nb, 1), 0);
-        int64_t ptot = 0;
+        double work = 0;  // complex products of phase 1
+        for (int i = 0; i < nb; ++i) {
+            const auto& b = op.blocks[i];
+            if (b.rank == 0) continue;
+            work += (double)b.rank * b.n;
+            cls[{(long long)b.rh_off, op.block_prob.empty() ? 0 : op.block_prob[i]}].push_back(i);
+        }
+        // a segment of R (64 rows, 16 columns) is at most about a
+        // sixteenth of an SM's share of the work, between 128 and 512 columns:
+        // shorter ones on small operators, where one long item would be the last
+        // to finish (12 x 12 array of 3^3 cubes in float64: 1.77 ms with 512)
+        op.tile_seg = 128;
+        while (op.tile_seg < 512 && 2.0 * op.tile_seg * 64 * 16 * 16 * op.ctx->n_sm <= work) op.tile_seg *= 2;
+        const int seg_len = op.tile_seg;
+        std::vector<long long> poff(std::max(nb, 1), 0), ctoff(std::max(nb, 1), 0);
+        std::vector<int> cseg;
+        int64_t ptot = 0, ctot = 0;
         for (int i = 0; i < nb; ++i) {
             const auto& b = op.blocks[i];
             poff[i] = ptot;
+            ctoff[i] = ctot;
             if (b.rank == 0) continue;
             ptot += (int64_t)b.nt * op.np;
-            cls[{(long long)b.rh_off, op.block_prob.empty() ? 0 : op.block_prob[i]}].push_back(i);
+            ctot += (int64_t)b.rank * ((b.n + seg_len - 1) / seg_len);
+            if (b.n > seg_len) cseg.push_back(i);
         }
         std::vector<int> cmem;
-        std::vector<int4> c1, c2;
-        std::vector<double> v1, v2;
+        std::vector<FarTile> c1, c2;
         int64_t nmem = 0;
+        op.tile_group = 1;
         for (const auto& kv : cls) {
             const auto& mem = kv.second;
             nmem += (int64_t)mem.size();
             const auto& b = op.blocks[mem[0]];
-            const size_t G = Op::kShareGroup;
-            for (size_t g = 0; g < mem.size(); g += G) {
+            auto tiles = [](int rows, int most, auto&& f) {  // equal pieces of at most `most` rows
+                const int nt = (rows + most - 1) / most, per = ((rows + nt - 1) / nt + 1) / 2 * 2;  // even: 16-byte copies
+                for (int r0 = 0; r0 < rows; r0 += per) f(r0, std::min(per, rows - r0));
+            };
+            for (size_t g = 0; g < mem.size(); g += kTileMembers) {
                 const int first = (int)cmem.size();
-                const int cnt = (int)std::min<size_t>(G, mem.size() - g);
+                const int cnt = (int)std::min<size_t>(kTileMembers, mem.size() - g);
+                op.tile_group = std::max(op.tile_group, cnt);
                 for (int j = 0; j < cnt; ++j) cmem.push_back(mem[g + j]);
-                for (int k0 = 0; k0 < b.rank; k0 += 32) {
-                    const int k1 = std::min(b.rank, k0 + 32);
-                    c1.push_back(make_int4(first, k0, k1, cnt));
-                    v1.push_back((double)(k1 - k0) * b.n * (1.0 + 0.25 * cnt));
-                }
-                for (int sl = 0; sl < b.nt; ++sl)
-                    for (int p0 = 0; p0 < op.np; p0 += 128) {
-                        const int p1e = std::min(op.np, p0 + 128);
-                        c2.push_back(make_int4(first, sl, p0 | (p1e << 16), cnt));
-                        v2.push_back((double)(p1e - p0) * b.rank * (1.0 + 0.25 * cnt));
-                    }
+                for (int seg = 0; seg * seg_len < b.n; ++seg)
+                    tiles(b.rank, 64, [&](int r0, int rows) {
+                        c1.push_back(FarTile{first, cnt, r0, rows, seg * seg_len, std::min(b.n, (seg + 1) * seg_len),
+                                             seg, 0});
+                    });
+                tiles(b.m, 256, [&](int r0, int rows) { c2.push_back(FarTile{first, cnt, r0, rows, 0, 0, 0, 0}); });
             }
         }
         op.share_mean = cls.empty() ? 1.0 : (double)nmem / (double)cls.size();
         op.part_total = ptot;
-        op.n_cta_c = op.ctx->n_sm * 3;
-        std::vector<int4> q1, q2;
-        std::vector<int> e1, e2;
-        pack_lpt(c1, v1, op.n_cta_c, q1, e1);
-        pack_lpt(c2, v2, op.n_cta_c, q2, e2);
-        op.n_c1_items = (int)q1.size();
-        op.n_c2_items = (int)q2.size();
-        upload(op.d_c1_items, q1.empty() ? std::vector<int4>{make_int4(0, 0, 0, 0)} : q1);
-        upload(op.d_c1_cta, e1);
-        upload(op.d_c2_items, q2.empty() ? std::vector<int4>{make_int4(0, 0, 0, 0)} : q2);
-        upload(op.d_c2_cta, e2);
+        op.ct_total = ctot;
+        op.n_c1_items = (int)c1.size();
+        op.n_c2_items = (int)c2.size();
+        upload(op.d_c1_items, c1.empty() ? std::vector<FarTile>{FarTile{}} : c1);
+        upload(op.d_c2_items, c2.empty() ? std::vector<FarTile>{FarTile{}} : c2);
+        op.n_cseg = (int)cseg.size();
+        upload(op.d_cseg, cseg);
         upload(op.d_cmem, cmem.empty() ? std::vector<int>{0} : cmem);
         upload(op.d_poff, poff);
-        op.d_part.release();  // sized on first use (shared_reserve)
+        upload(op.d_ctoff, ctoff);
+        op.d_part.release();  // sized on first use (tile_reserve)
+        op.d_ct.release();
     }
 }
 

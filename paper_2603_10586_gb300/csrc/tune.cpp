@@ -1,9 +1,9 @@
 // Far-apply variants and the autotuner that chooses between them.
 //
 // The far part of a complex float32 apply has several implementations: the
-// SIMT kernels with 1, 2, 4 or 8 right-hand sides per factor read (register
-// tiles), the SIMT kernels that apply translated copies of a block together
-// (one factor read per group of copies), and for split-precision requests the
+// SIMT kernels with 1, 2, 4 or 8 right-hand sides per factor read, the
+// register-tile kernels over the columns (translated copies x right-hand sides)
+// of a factor, and for split-precision requests the
 // warp-MMA and the tcgen05 tensor-core kernels.  Which is fastest depends on the right-hand-side count
 // and on the operator (rank distribution, atom size), so the choice is made by
 // timing on the operator itself and is remembered per power-of-two bucket of
@@ -31,9 +31,6 @@ bool admissible(int precision, int v) {
 }
 
 int default_variant(const Op& op, int precision, int nrhs) {
-    // one right-hand side: read shared factors once per group of copies when
-    // the operator has translated copies
-    if (nrhs == 1) return op.share_mean > 1.5 ? VIE_VAR_SIMT_SHARED : VIE_VAR_SIMT_R1;
     // BF16x3: the warp-specialised kernel with one row tile per B tile streams
     // the A planes fastest while the B operand is narrow (8.6 ms per apply of
     // the 32 x 32 array of 4^3 cubes at 16 columns); wider, the gathers of B
@@ -41,7 +38,17 @@ int default_variant(const Op& op, int precision, int nrhs) {
     // 48 / 64 columns, against 11.2 / 16.4 / 19.8 ms)
     if (precision == VIE_BF16X3 && nrhs >= 8)
         return nrhs <= 16 ? VIE_VAR_TCGEN05_WS_BF16X3 : VIE_VAR_TCGEN05_WS2_BF16X3;
-    return VIE_VAR_SIMT_R4;
+    return nrhs == 1 ? (tile_pays(op, 1) ? VIE_VAR_SIMT_SHARED : VIE_VAR_SIMT_R1) : VIE_VAR_SIMT_R4;
+}
+
+// the variants that read a factor once per group of right-hand sides: the
+// register tiles take all columns (copies x right-hand sides) of a factor
+// together where that pays, in one summation order for the three group sizes
+void far_grouped(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, int nr, cudaStream_t s) {
+    if (tile_pays(op, nrhs) && tile_reserve(op, nrhs, sizeof(float2), s))
+        apply_far_tile<float2, float2, float2>(op, x, ldx, F, ldf, nrhs, s);
+    else
+        apply_far_simt32(op, x, ldx, F, ldf, nrhs, nr, s);
 }
 
 }  // namespace
@@ -54,13 +61,21 @@ int far_variant(const Op& op, int precision, int nrhs) {
 void far32(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, int precision, cudaStream_t s) {
     switch (far_variant(op, precision, nrhs)) {
         case VIE_VAR_SIMT_R1: apply_far_simt32(op, x, ldx, F, ldf, nrhs, 1, s); break;
-        case VIE_VAR_SIMT_R2: apply_far_simt32(op, x, ldx, F, ldf, nrhs, 2, s); break;
-        case VIE_VAR_SIMT_R4: apply_far_simt32(op, x, ldx, F, ldf, nrhs, 4, s); break;
-        case VIE_VAR_SIMT_R8: apply_far_simt32(op, x, ldx, F, ldf, nrhs, 8, s); break;
+        case VIE_VAR_SIMT_R2: far_grouped(op, x, ldx, F, ldf, nrhs, 2, s); break;
+        case VIE_VAR_SIMT_R4: far_grouped(op, x, ldx, F, ldf, nrhs, 4, s); break;
+        case VIE_VAR_SIMT_R8: far_grouped(op, x, ldx, F, ldf, nrhs, 8, s); break;
         case VIE_VAR_MMA_BF16X3: apply_far_bf16x3(op, x, ldx, F, ldf, nrhs, s); break;
         case VIE_VAR_TCGEN05_BF16X3: apply_far_umma(op, x, ldx, F, ldf, nrhs, s); break;
         case VIE_VAR_TCGEN05_PACKED_BF16X3: apply_far_umma_packed(op, x, ldx, F, ldf, nrhs, s); break;
-        case VIE_VAR_SIMT_SHARED: apply_far_shared(op, x, ldx, F, ldf, nrhs, s); break;
+        case VIE_VAR_SIMT_SHARED:
+            // one right-hand side at a time: a column's result does not depend on the others
+            for (int c = 0; c < nrhs; ++c) {
+                if (tile_reserve(op, 1, sizeof(float2), s))
+                    apply_far_tile<float2, float2, float2>(op, x, ldx, F, ldf, nrhs, s, c, 1);
+                else
+                    apply_far_simt32(op, x + c * ldx, ldx, F + c * ldf, ldf, 1, 1, s);
+            }
+            break;
         case VIE_VAR_TCGEN05_WS_BF16X3: apply_far_umma_ws(op, x, ldx, F, ldf, nrhs, s); break;
         case VIE_VAR_TCGEN05_WS2_BF16X3: apply_far_umma_ws2(op, x, ldx, F, ldf, nrhs, s); break;
         default: fail(VIE_ERR_STATE, "unknown far-apply variant");
