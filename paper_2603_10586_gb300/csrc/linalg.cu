@@ -6,6 +6,7 @@
 // operator, the preconditioner and the fused P^-1 Z form).
 #include "common.h"
 #include "cplx.cuh"
+#include "tilemma.cuh"
 
 namespace vie {
 
@@ -156,73 +157,125 @@ __global__ void c64_to_c128(const float2* s, double2* d, int64_t n) {
 // ---------------------------------------------------------------------------
 // Y[:, col] = M B[:, col] (+ ADD[:, col]) for the columns col = (atom of the
 // type, rhs).  M: np x np column-major.  Vector element (row r of atom a, rhs c)
-// lives at a * np + r + c * ld.  32 x 32 output tile per CTA (enough CTAs for a
-// few hundred atoms), 256 threads, each a 2 x 2 sub-tile; K staged through
-// shared memory 32 at a time.
+// lives at a * np + r + c * ld.  A CTA of four warps takes 16 RA rows x 2 J WN
+// columns, the warps side by side and, where the columns are few, along K (WK =
+// 4 / WN groups added in order at the end); operands staged by cp.async through two
+// shared-memory buffers.  Bound by the float32 (float64) pipes; the launcher picks
+// the widest tile that still fills the GPU twice over.  (A 2 x 2 sub-tile per
+// thread and 32 x 32 per CTA, the kernel before, took 997 us for 61,440 columns of
+// np = 240 in float32, now 669 us, and 19 us for 16 columns of np = 108, now 9 us.)
 // ADD may be Y itself (y = Z_ii x + y in place): every output element is read
 // from ADD and then written to Y by the one thread that owns it, so ADD and Y
 // carry no __restrict__ and ADD is read through the ordinary (coherent) path.
 // B must not overlap Y.
 // ---------------------------------------------------------------------------
-template <class TM, class TX>
-__global__ void __launch_bounds__(256) type_gemm(const TM* __restrict__ M, int np, const int* __restrict__ atoms,
-                                                 int n_atoms, int nrhs, const TX* __restrict__ B, int64_t ldb,
-                                                 const TX* ADD, int64_t ldadd, TX* Y, int64_t ldy,
-                                                 const int2* __restrict__ colr, int prob) {
-    using R = decltype(TM().x);
-    using TA = typename C2<R>::t;
-    constexpr int BM = 32, BN = 32, BK = 32;
-    __shared__ TA sM[BK][BM + 1];
-    __shared__ TA sB[BK][BN + 1];
+constexpr int kGemmThr = 128;
+template <class T, int WN, int RA, int J>
+struct GemmShape {
+    static constexpr int WK = 4 / WN, TM = 16 * RA, TN = 2 * J * WN;
+    static constexpr int KC = 16, KG = KC / WK;
+    static constexpr int LA = TM, LB = KC + kE<T>;  // A [K][row], B [column][K]
+    static constexpr size_t a_pad = (size_t)KC * LA * sizeof(T);
+    static constexpr size_t stage = a_pad + (size_t)TN * LB * sizeof(T);
+};
+
+template <class T, int WN, int RA, int J>
+__global__ void __launch_bounds__(kGemmThr, 3) type_gemm(const T* __restrict__ M, int np, int tile_rows,
+                                                         const int* __restrict__ atoms, int n_atoms, int nrhs,
+                                                         const T* __restrict__ B, int64_t ldb, const T* ADD,
+                                                         int64_t ldadd, T* Y, int64_t ldy,
+                                                         const int2* __restrict__ colr, int prob) {
+    using S = GemmShape<T, WN, RA, J>;
+    constexpr int E = kE<T>, UR = S::TM / E, UK = S::KC / E;   // 16-byte units per K value of A, per column of B
+    constexpr int KA = kGemmThr / UR, CB = kGemmThr / UK;      // K values of A, columns of B staged at a time
+    constexpr int NB = (S::TN + CB - 1) / CB;
+    __shared__ __align__(16) unsigned char smem[2 * S::stage];
     // right-hand sides of this type's problem (all of them for a single operator)
     const int2 cr = colr ? colr[prob] : make_int2(0, nrhs);
     const int ncols = n_atoms * (cr.y - cr.x);
-    const int row0 = blockIdx.x * BM, col0 = blockIdx.y * BN;
+    const int row0 = blockIdx.x * tile_rows, rows = min(tile_rows, np - row0), col0 = blockIdx.y * S::TN;
     if (col0 >= ncols) return;
-    const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;  // 16 x 16 threads, 2 x 2 each
-    TA acc[2][2];
-    for (int a = 0; a < 2; ++a)
-        for (int b = 0; b < 2; ++b) acc[a][b] = mk(R(0), R(0));
-    // column -> (atom, rhs) base offsets for the B loads of this tile
-    for (int k0 = 0; k0 < np; k0 += BK) {
-        for (int e = threadIdx.x; e < BK * BM; e += 256) {
-            int kk = e / BM, r = e % BM;
-            int gr = row0 + r, gk = k0 + kk;
-            sM[kk][r] = (gr < np && gk < np) ? cvt<TA>(M[gr + (int64_t)gk * np]) : mk(R(0), R(0));
-        }
-        for (int e = threadIdx.x; e < BK * BN; e += 256) {
-            int kk = e % BK, c = e / BK;
-            int gc = col0 + c, gk = k0 + kk;
-            TA v = mk(R(0), R(0));
-            if (gc < ncols && gk < np) {
-                int a = atoms[gc % n_atoms], rhs = cr.x + gc / n_atoms;
-                v = cvt<TA>(B[(int64_t)a * np + gk + (int64_t)rhs * ldb]);
-            }
-            sB[kk][c] = v;
-        }
-        __syncthreads();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int wn = warp % WN, wk = warp / WN, tr = lane & 15, tc = lane >> 4;
+    const int ur = tid % UR * E, uk = tid / UR, kb = tid % UK * E, cb = tid / UK;
+    const T* Ms = M + row0 + ur + (int64_t)uk * np;
+    const T* bs[NB];
+    unsigned live = 0;
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            TA mv[2], bv[2];
-            for (int a = 0; a < 2; ++a) mv[a] = sM[kk][tr + 16 * a];
-            for (int b = 0; b < 2; ++b) bv[b] = sB[kk][tc + 16 * b];
-            for (int a = 0; a < 2; ++a)
-                for (int b = 0; b < 2; ++b) cfma(acc[a][b], mv[a], bv[b]);
+    for (int u = 0; u < NB; ++u) {
+        const int q = cb + u * CB, gc = col0 + q;
+        const bool ok = q < S::TN && gc < ncols;
+        bs[u] = ok ? B + (int64_t)atoms[gc % n_atoms] * np + kb + (int64_t)(cr.x + gc / n_atoms) * ldb : B;
+        live |= ok ? 1u << u : 0u;
+    }
+    const int nst = (np + S::KC - 1) / S::KC;
+    auto fill = [&](int s) {
+        T* As = reinterpret_cast<T*>(smem + (s & 1) * S::stage) + uk * S::LA + ur;
+        T* Bs = reinterpret_cast<T*>(smem + (s & 1) * S::stage + S::a_pad) + cb * S::LB + kb;
+#pragma unroll
+        for (int k = 0; k < S::KC; k += KA) {
+            const bool ok = s * S::KC + k + uk < np && ur < rows;
+            if (KA <= S::KC || uk < S::KC)
+                cp_async16(As + k * S::LA, ok ? Ms + (int64_t)(s * S::KC + k) * np : M, ok);
+        }
+#pragma unroll
+        for (int u = 0; u < NB; ++u)
+            if (cb + u * CB < S::TN) {
+                const bool ok = ((live >> u) & 1) && s * S::KC + kb < np;
+                cp_async16(Bs + u * CB * S::LB, ok ? bs[u] + s * S::KC : B, ok);
+            }
+        cp_commit();
+    };
+    T acc[RA][J];
+    zero_acc(acc);
+    fill(0);
+    for (int s = 0; s < nst; ++s) {
+        if (s + 1 < nst) {
+            fill(s + 1);
+            cp_wait<1>();
+        } else {
+            cp_wait<0>();
         }
         __syncthreads();
+        const unsigned char* st = smem + (s & 1) * S::stage;
+        mma_stage<T, T, T, 2, S::KG, S::LA, S::LB, RA, J>(
+            reinterpret_cast<const T*>(st) + wk * S::KG * S::LA + E * tr,
+            reinterpret_cast<const T*>(st + S::a_pad) + (wn * 2 * J + tc) * S::LB + wk * S::KG, acc);
+        __syncthreads();
     }
-    for (int b = 0; b < 2; ++b) {
-        int gc = col0 + tc + 16 * b;
-        if (gc >= ncols) continue;
-        int a_ = atoms[gc % n_atoms], rhs = cr.x + gc / n_atoms;
-        for (int a = 0; a < 2; ++a) {
-            int gr = row0 + tr + 16 * a;
-            if (gr >= np) continue;
-            TA v = acc[a][b];
-            if (ADD) v += cvt<TA>(ADD[(int64_t)a_ * np + gr + (int64_t)rhs * ldadd]);
-            Y[(int64_t)a_ * np + gr + (int64_t)rhs * ldy] = cvt<TX>(v);
+    if (S::WK > 1) {
+        T* buf = reinterpret_cast<T*>(smem);
+#pragma unroll
+        for (int g = 1; g < S::WK; ++g) {
+            if (wk == g)
+#pragma unroll
+                for (int i = 0; i < RA; ++i)
+#pragma unroll
+                    for (int j = 0; j < J; ++j) buf[((wn * RA + i) * J + j) * 32 + lane] = acc[i][j];
+            __syncthreads();
+            if (wk == 0)
+#pragma unroll
+                for (int i = 0; i < RA; ++i)
+#pragma unroll
+                    for (int j = 0; j < J; ++j) acc[i][j] += buf[((wn * RA + i) * J + j) * 32 + lane];
+            __syncthreads();
         }
     }
+    if (wk == 0)
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const int gc = col0 + wn * 2 * J + tc + 2 * j;
+            if (gc >= ncols) continue;
+            const int64_t at = (int64_t)atoms[gc % n_atoms] * np + row0, rhs = cr.x + gc / n_atoms;
+#pragma unroll
+            for (int i = 0; i < RA; ++i) {
+                const int r = E == 2 ? 32 * (i >> 1) + 2 * tr + (i & 1) : 16 * i + tr;
+                if (r >= rows) continue;
+                T v = acc[i][j];
+                if (ADD) v += ADD[at + r + rhs * ldadd];
+                Y[at + r + rhs * ldy] = v;
+            }
+        }
 }
 
 }  // namespace
@@ -310,6 +363,19 @@ void conj_transpose_blocks(const void* src, void* dst, int T, int np, bool c128,
     VIE_CHECK_LAUNCH();
 }
 
+namespace {
+template <class T, int WN, int RA, int J>
+void launch_gemm(const T* M, int np, const int* atoms, int na, int nrhs, const T* B, int64_t ldb, const T* ADD,
+                 int64_t ldadd, T* Y, int64_t ldy, const int2* colr, int prob, cudaStream_t s) {
+    using S = GemmShape<T, WN, RA, J>;
+    const int nt = (np + S::TM - 1) / S::TM, tile_rows = ((np + nt - 1) / nt + 1) / 2 * 2;  // equal, even pieces
+    const dim3 grid((np + tile_rows - 1) / tile_rows, (unsigned)(((int64_t)na * nrhs + S::TN - 1) / S::TN));
+    type_gemm<T, WN, RA, J><<<grid, kGemmThr, 0, s>>>(M, np, tile_rows, atoms, na, nrhs, B, ldb, ADD, ldadd, Y, ldy,
+                                                      colr, prob);
+    VIE_CHECK_LAUNCH();
+}
+}  // namespace
+
 // mode 0: Y = M X + C   (self part plus far part C)
 // mode 1: Y = X + M C   (fused preconditioner: X + Z_D^-1 (far part))
 // mode 2: Y = M X       (plain block product, e.g. the preconditioner)
@@ -317,19 +383,28 @@ template <class TM, class TX>
 void self_gemm(Op& op, const TM* M, const TX* X, int64_t ldx, const TX* C, int64_t ldc, TX* Y, int64_t ldy,
                int nrhs, int mode, cudaStream_t s) {
     const int np = op.np;
+    constexpr int J = sizeof(TX) == 8 ? 8 : 4;
     for (int t = 0; t < op.T; ++t) {
         int na = op.type_atom_off[t + 1] - op.type_atom_off[t];
         if (na == 0) continue;
         const int* atoms = op.d_atoms_by_type.as<int>() + op.type_atom_off[t];
         const TM* Mt = M + (size_t)t * np * np;
-        dim3 grid((np + 31) / 32, (na * nrhs + 31) / 32);
         const TX* Bop = mode == 1 ? C : X;
         int64_t ldb = mode == 1 ? ldc : ldx;
         const TX* ADD = mode == 0 ? C : (mode == 1 ? X : nullptr);
         int64_t ldadd = mode == 0 ? ldc : ldx;
         const int prob = op.type_prob.empty() ? 0 : op.type_prob[t];
-        type_gemm<TM, TX><<<grid, 256, 0, s>>>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob);
-        VIE_CHECK_LAUNCH();
+        // the widest tile that gives every SM two CTAs; the narrowest (32 rows, four
+        // warps along K) when none does
+        const int64_t rt = (np + 63) / 64, cols = (int64_t)na * nrhs, want = 2 * op.ctx->n_sm;
+        auto enough = [&](int tn) { return rt * ((cols + tn - 1) / tn) >= want; };
+#define VIE_GEMM(WN, RA) \
+    launch_gemm<TX, WN, RA, J>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s)
+        if (enough(8 * J)) VIE_GEMM(4, 4);
+        else if (enough(4 * J)) VIE_GEMM(2, 4);
+        else if (enough(2 * J)) VIE_GEMM(1, 4);
+        else launch_gemm<TX, 1, 2, 4>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s);
+#undef VIE_GEMM
     }
 }
 
