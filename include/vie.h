@@ -92,20 +92,21 @@ enum vie_variant {
                                element read once per group of up to 64 copies; partial products are
                                summed per target atom in a fixed order (default for one right-hand
                                side when the operator has translated copies) */,
-    VIE_VAR_TCGEN05_WS_BF16X3 = 9 /* the planes of 7 in a warp-specialised persistent kernel (one CTA
-                                     per SM): a warp moves the A planes by bulk TMA into a ring of 3 to
-                                     5 stages (5 up to 16 right-hand sides, 4 up to 48), up to four warp
-                                     pairs gather and split B into two stacked plane sets, one thread
-                                     issues four wide MMAs per K step (each A plane read once), four
-                                     warps drain two tensor-memory accumulator buffers; equal to 7 to
-                                     float32 rounding (default for 8 to 16 right-hand sides; runs as 6
-                                     when the planes do not fit) */,
+    VIE_VAR_TCGEN05_WS_BF16X3 = 9 /* the factors split once into bf16 planes, held once per factor
+                                     storage (translated copies share them), in a warp-specialised
+                                     persistent kernel (one CTA per SM): a warp moves the A planes by bulk
+                                     TMA into a ring of 3 to 5 stages (5 up to 16 right-hand sides, 4 up to
+                                     48), up to four warp pairs gather and split B into two stacked plane
+                                     sets, a warp issues four wide MMAs per K step (each A plane read
+                                     once), four warps drain two tensor-memory accumulator buffers; equal
+                                     to 7 to float32 rounding (default for 8 to 32 right-hand sides on
+                                     atoms of at most 128 unknowns; runs as 6 when the planes do not fit) */,
     VIE_VAR_TCGEN05_WS2_BF16X3 = 10 /* 9 with two 128-row tiles of factor rows sharing each B tile (the
                                        two row tiles of a target atom, or two consecutive row tiles of
                                        a source group), 16 K values per stage: the B operand is gathered
                                        and split once for twice the rows; equal to 9 to float32
-                                       rounding (default for more than 16 right-hand sides; runs as 6
-                                       when the planes do not fit) */
+                                       rounding (default for 8 right-hand sides or more otherwise; runs
+                                       as 6 when the planes do not fit) */
 };
 
 /* vie_apply flags */
@@ -159,9 +160,9 @@ typedef struct vie_op_info {
     double t_assemble_s, t_compress_s;
     int64_t stored_entries;    /* factor entries held in memory: translated copies of a far block
                                   share one set of factors (see vie_ctx_opts.no_sharing) */
-    int64_t packed_bytes;      /* bytes of the bf16 planes the packed tensor-core apply streams per
-                                  application (every far block's own planes, tiles padded to 128 rows
-                                  and K to 32); 0 until a VIE_BF16X3 apply has built them */
+    int64_t packed_bytes;      /* bytes of the bf16 planes the tensor-core apply holds (one set per factor
+                                  storage, ranks padded to 8, atoms to 128 rows); 0 until a VIE_BF16X3
+                                  apply has built them */
     int compress_method;       /* vie_compress_method of the stored factors */
     double cross_bytes;        /* cross approximation: residual bytes its passes read and wrote */
     double t_cross_s;          /* cross approximation: device time of its step loops */

@@ -87,8 +87,21 @@ void op_apply_fused64(Op& op, const double2* x, double2* y, int nrhs, cudaStream
 
 void op_reserve(Op& op, int nrhs, int precision, cudaStream_t s) {
     if (precision == VIE_BF16X3) {
-        umma_prepare(op, s);
-        umma_pack(op, s);  // any cycle's right-hand-side count may choose the packed variant
+        // what any cycle's right-hand-side count may choose: the warp-specialised
+        // kernels from 8 columns on, or a tuned variant
+        bool ws = false, plain = false, packed = false;
+        for (int k = 1; k <= nrhs; ++k) {
+            const int v = far_variant(op, precision, k);
+            ws |= v == VIE_VAR_TCGEN05_WS_BF16X3 || v == VIE_VAR_TCGEN05_WS2_BF16X3;
+            plain |= v == VIE_VAR_TCGEN05_BF16X3;
+            packed |= v == VIE_VAR_TCGEN05_PACKED_BF16X3;
+        }
+        if (ws) {
+            if (ws_pack(op, s)) ws_reserve(op, nrhs);
+            else plain = true;
+        }
+        if (packed) umma_pack(op, s);
+        if (plain || packed) umma_prepare(op, s);
     }
     ensure_F(op, (size_t)op.n() * nrhs * sizeof(double2));
     const size_t need = (size_t)std::max<int64_t>(op.t_total, 1) * nrhs * sizeof(double2);
@@ -403,7 +416,7 @@ int vie_op_get_info(const vie_op* op, vie_op_info* info) {
     info->t_assemble_s = o.t_assemble;
     info->t_compress_s = o.t_compress;
     info->stored_entries = o.stored_entries;
-    info->packed_bytes = o.umma_packed ? (int64_t)umma_pack_bytes(o) : 0;
+    info->packed_bytes = o.ws_packed ? (int64_t)ws_plane_bytes(o) : o.umma_packed ? (int64_t)umma_pack_bytes(o) : 0;
     info->compress_method = o.cmethod;
     info->cross_bytes = o.cross_bytes;
     info->t_cross_s = o.t_cross;

@@ -204,14 +204,18 @@ struct Op {
     // the SIMT lists mapped to two CTAs per SM (the multi-RHS SIMT kernels)
     int n_cta_m = 0;
     DevBuf d_p1m_items, d_p1m_cta, d_p2m_items, d_p2m_cta;
-    DevBuf d_w1_items, d_w1_cta, d_w1_pk, d_w2_items, d_w2_cta, d_w2_pk;  // one CTA per SM (warp-specialised)
-    // pairs of items that share their B operand (two M tiles per B tile), one CTA per SM: first and
-    // second item (rows 0 when absent) and their packed stage offsets
-    DevBuf d_x1_items, d_x1_items_b, d_x1_cta, d_x1_pk, d_x1_pk_b;
-    DevBuf d_x2_items, d_x2_items_b, d_x2_cta, d_x2_pk, d_x2_pk_b;
     long long u1_stages = 0, u2_stages = 0;
     bool umma_packed = false, umma_pack_failed = false;
     int n_u1_items = 0, n_u2_items = 0, n_cta_u = 0;
+    // warp-specialised variants (apply_ws.cu): the factors' bf16 planes once per
+    // factor storage, item lists per tile shape ([0] one, [1] two row tiles per B
+    // tile), phase 1 runs and t places of the stacked 8-row groups, phase 2 chunks
+    // per atom
+    bool ws_ready = false, ws_packed = false, ws_pack_failed = false;
+    int ws_ncls = 0, n_ws1[2] = {0, 0};
+    int64_t ws_r_units = 0, ws_q_chunks = 0, ws_t_total = 0;
+    DevBuf d_ws_cls, d_ws_r, d_ws_q, d_ws_grp, d_ws_kptr, d_ws_qidx, d_ws_tidx;
+    DevBuf d_ws1_items[2], d_ws1_cta[2], d_ws_runs[2], d_ws2_items[2], d_ws2_cta[2];
     DevBuf d_err;  // set by a tensor-core kernel whose bounded wait gave up
     // batched operators (several problems as one block-diagonal operator,
     // batch.cpp): problem of every block, atom and type, and during a solve
@@ -283,6 +287,53 @@ struct FarTile {
     int first, nm, row0, rows, k0, k1, seg, pad;
 };
 constexpr int kTileMembers = 64;  // members per item: a full group fills 64-column tiles whatever the right-hand-side count
+
+// ---- warp-specialised tensor-core apply (apply_ws.cu) -----------------------
+// planes of one factor storage: R as 1 KB units (16 K values x 8 rows) from
+// r_unit on, [K unit][row group]; Q as 8 KB chunks (8 K values x 128 rows of a
+// slot) from q_chunk on, [slot][K chunk], one such region per row tile
+struct WsClass {
+    long long rh_off, q_off, r_unit, q_chunk;
+    int rank, n, m, pad;
+};
+// phase 1: consecutive 8-row groups of one block inside a 128-row tile: first
+// unit at K unit 0, units per K unit, group in the tile, groups
+struct WsRun {
+    long long unit;
+    int step, g0, ng, pad;
+};
+// phase 1 item: one or two 128-row tiles of a source group's stacked rows (rep:
+// a block with that source; grp0: the first stacked group, 16 per tile)
+struct WsItem1 {
+    int rep, prob, grp0, run0, nrun[2], ngrp[2];
+};
+// phase 2 item: one or two row tiles (from rt on) of an atom
+struct WsItem2 {
+    int atom, prob, rt, rows[2];
+};
+struct FarBlockDev;
+struct WsArgs1 {
+    const FarBlockDev* blocks;
+    const int* batoms;
+    const WsItem1* items;
+    const int* cta_ptr;
+    const WsRun* runs;
+    const int* grp_t;
+    const unsigned char* planes;
+    const float2* x8;
+    int64_t ldx;
+    int per, nrhs;
+    const int2* colr;
+};
+struct WsArgs2 {
+    const WsItem2* items;
+    const int *cta_ptr, *kptr, *qidx, *tidx;
+    const unsigned char* planes;
+    const float2* t;
+    int64_t ldt, rt_bytes;  // values per chunk of t, bytes of a row tile's planes
+    int np, nrhs;
+    const int2* colr;
+};
 
 // device-side block description used by the apply kernels
 struct FarBlockDev {
@@ -378,6 +429,12 @@ void umma_prepare(Op& op, cudaStream_t s);
 bool umma_pack(Op& op, cudaStream_t s);
 size_t umma_pack_bytes(const Op& op);
 void apply_far_umma_packed(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
+// warp-specialised variants: lists (host.cpp), planes (false when the free memory
+// cannot hold them; the unpacked kernel runs instead), scratch for nrhs columns
+void build_ws_lists(Op& op);
+bool ws_pack(Op& op, cudaStream_t s);
+void ws_reserve(Op& op, int nrhs);
+size_t ws_plane_bytes(const Op& op);
 void apply_far_umma_ws(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
 void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s);
 // apply_tile.cu: far apply by register tiles over classes of blocks that share

@@ -8,6 +8,7 @@
 #include <map>
 #include <numeric>
 #include <queue>
+#include <unordered_map>
 
 #include "common.h"
 
@@ -268,10 +269,8 @@ static void pack_lpt(const std::vector<int4>& items, const std::vector<double>& 
 // Load of one tensor-core tile in K stages: every stage moves the same bytes
 // (A planes padded to 128 rows) and takes the same MMAs whatever the tile's
 // real row count, so the rows do not enter; a tile also pays its accumulator
-// drain, about two stages.  A pair of row tiles (the paired-tile kernels, 16
-// K values per stage) costs twice the stages of its first tile.
+// drain, about two stages.
 static double tile_cost(int64_t K, int ks) { return (double)((K + ks - 1) / ks) + 2.0; }
-static double pair_cost(double single32) { return 2.0 * (single32 - 2.0) + 2.0; }
 
 // Z-order (Morton) code of every atom centre, from its x, y position in the
 // array's bounding box quantised to 16 bits per axis
@@ -419,6 +418,9 @@ void build_apply_lists(Op& op) {
     upload(op.d_p2_csr, csr);
     upload(op.d_p2_ent, flat.empty() ? std::vector<int2>{make_int2(0, 0)} : flat);
     op.umma_ready = false;
+    op.ws_ready = op.ws_packed = op.ws_pack_failed = false;
+    op.d_ws_r.release();
+    op.d_ws_q.release();
 
     // register-tile path: classes of blocks with the same factor storage, in
     // groups of up to kTileMembers members; phase 1 items of up to 64 rows and
@@ -563,13 +565,10 @@ void build_umma_lists(Op& op) {
             key2.push_back(zc[a]);
         }
     }
-    std::vector<int4> q1, q2, r1, r2;
-    std::vector<int> e1, e2, f1, f2, p1, p2, pr1, pr2;
+    std::vector<int4> q1, q2;
+    std::vector<int> e1, e2, p1, p2;
     pack_lpt(it1, w1, op.n_cta_u, q1, e1, &p1, &key1);
     pack_lpt(it2, w2, op.n_cta_u, q2, e2, &p2, &key2);
-    // the same items mapped to one CTA per SM (warp-specialised kernels)
-    pack_lpt(it1, w1, op.ctx->n_sm, r1, f1, &pr1, &key1);
-    pack_lpt(it2, w2, op.ctx->n_sm, r2, f2, &pr2, &key2);
     op.n_u1_items = (int)q1.size();
     op.n_u2_items = (int)q2.size();
     upload(op.d_u1_rowoff, rowoff.empty() ? std::vector<long long>{0} : rowoff);
@@ -594,75 +593,155 @@ void build_umma_lists(Op& op) {
     op.u2_stages = pk2.back();
     upload(op.d_u1_pk, pk1);
     upload(op.d_u2_pk, pk2);
-    // stage offsets of the one-CTA-per-SM lists: the planes stay where the
-    // first list put them (item i of that list at pk[i])
-    auto remap = [](const std::vector<int>& perm_from, const std::vector<int>& perm_to,
-                    const std::vector<long long>& pk) {
-        std::vector<int> pos(perm_from.size());
-        for (size_t i = 0; i < perm_from.size(); ++i) pos[perm_from[i]] = (int)i;
-        std::vector<long long> out(perm_to.size() + 1, pk.back());
-        for (size_t i = 0; i < perm_to.size(); ++i) out[i] = pk[pos[perm_to[i]]];
-        return out;
-    };
-    upload(op.d_w1_items, r1.empty() ? std::vector<int4>{make_int4(0, 0, 0, 0)} : r1);
-    upload(op.d_w1_cta, f1);
-    upload(op.d_w1_pk, remap(p1, pr1, pk1));
-    upload(op.d_w2_items, r2.empty() ? std::vector<int4>{make_int4(0, 0, 0, 0)} : r2);
-    upload(op.d_w2_cta, f2);
-    upload(op.d_w2_pk, remap(p2, pr2, pk2));
-    // pairs of items with one B operand (the paired-tile kernels): two
-    // consecutive row tiles of one source group (phase 1) or of one target
-    // atom (phase 2); a leftover tile goes alone, its second item with 0 rows
-    auto pair_lists = [&](const std::vector<int4>& items, const std::vector<double>& w,
-                          const std::vector<uint64_t>& key, const std::vector<int>& perm_from,
-                          const std::vector<long long>& pk, auto same_b, auto empty_of, DevBuf& d_items,
-                          DevBuf& d_items_b, DevBuf& d_cta, DevBuf& d_pk, DevBuf& d_pk_b) {
-        std::vector<int> pos(perm_from.size());
-        for (size_t i = 0; i < perm_from.size(); ++i) pos[perm_from[i]] = (int)i;
-        std::vector<int2> pairs;
-        std::vector<int4> first;
-        std::vector<double> pw;
-        std::vector<uint64_t> pkey;
-        for (size_t i = 0; i < items.size(); ++i) {
-            const bool two = i + 1 < items.size() && same_b(items[i], items[i + 1]);
-            pairs.push_back(make_int2((int)i, two ? (int)i + 1 : -1));
-            first.push_back(items[i]);
-            pw.push_back(pair_cost(w[i]));
-            pkey.push_back(key[i]);
-            if (two) ++i;
-        }
-        std::vector<int4> out;
-        std::vector<int> cta, perm;
-        pack_lpt(first, pw, op.ctx->n_sm, out, cta, &perm, &pkey);
-        std::vector<int4> ib(out.size());
-        std::vector<long long> pa(out.size() + 1, pk.back()), pb(out.size() + 1, 0);
-        for (size_t k = 0; k < out.size(); ++k) {
-            const int2 pr = pairs[perm[k]];
-            pa[k] = pk[pos[pr.x]];
-            ib[k] = pr.y >= 0 ? items[pr.y] : empty_of(items[pr.x]);
-            pb[k] = pr.y >= 0 ? pk[pos[pr.y]] : 0;
-        }
-        upload(d_items, out.empty() ? std::vector<int4>{make_int4(0, 0, 0, 0)} : out);
-        upload(d_items_b, ib.empty() ? std::vector<int4>{make_int4(0, 0, 0, 0)} : ib);
-        upload(d_cta, cta);
-        upload(d_pk, pa);
-        upload(d_pk_b, pb);
-    };
-    // phase 1 items (rep block, first row, rows, problem); phase 2 (atom, p0, p1, problem)
-    pair_lists(
-        it1, w1, key1, p1, pk1,
-        [](const int4& a, const int4& b) { return a.x == b.x && b.y == a.y + a.z; },
-        [](const int4& a) { return make_int4(a.x, a.y, 0, a.w); }, op.d_x1_items, op.d_x1_items_b, op.d_x1_cta,
-        op.d_x1_pk, op.d_x1_pk_b);
-    pair_lists(
-        it2, w2, key2, p2, pk2, [](const int4& a, const int4& b) { return a.x == b.x && b.y == a.z; },
-        [](const int4& a) { return make_int4(a.x, 0, 0, a.w); }, op.d_x2_items, op.d_x2_items_b, op.d_x2_cta,
-        op.d_x2_pk, op.d_x2_pk_b);
     op.umma_packed = false;
     op.umma_pack_failed = false;
     op.d_u1_pack.release();
     op.d_u2_pack.release();
     op.umma_ready = true;
+}
+
+// Lists of the warp-specialised kernels (apply_ws.cu has the plane layouts).
+void build_ws_lists(Op& op) {
+    if (op.ws_ready) return;
+    const int nb = (int)op.blocks.size();
+    const int nrt = (op.np + 127) / 128, n_cta = op.ctx->n_sm;
+    const int per = (op.np + 7) / 8;  // chunks of 8 unknowns per atom (K axis of phase 1)
+    // factor storages and where their planes lie
+    std::vector<WsClass> cls;
+    std::vector<int> cls_of(nb, -1), t0(nb, 0);
+    std::unordered_map<long long, int> at;
+    op.ws_r_units = op.ws_q_chunks = op.ws_t_total = 0;
+    for (int i = 0; i < nb; ++i) {
+        const auto& b = op.blocks[i];
+        if (b.rank == 0) continue;
+        const int G = (b.rank + 7) / 8;
+        t0[i] = (int)(op.ws_t_total / 8);  // in units of 8 entries
+        op.ws_t_total += 8 * G;
+        const auto ins = at.emplace((long long)b.rh_off, (int)cls.size());
+        if (ins.second) {
+            cls.push_back(WsClass{(long long)b.rh_off, (long long)b.q_off, op.ws_r_units, op.ws_q_chunks, b.rank, b.n,
+                                  b.m, 0});
+            op.ws_r_units += (int64_t)((b.ns * per + 1) / 2) * G;
+            op.ws_q_chunks += (int64_t)b.nt * G;
+        }
+        cls_of[i] = ins.first->second;
+    }
+    if (op.ws_t_total > std::numeric_limits<int>::max() || op.ws_q_chunks > std::numeric_limits<int>::max())
+        fail(VIE_ERR_STATE, "the operator is too large for the warp-specialised apply's 32-bit places");
+    op.ws_ncls = (int)cls.size();
+    upload(op.d_ws_cls, cls.empty() ? std::vector<WsClass>{WsClass{}} : cls);
+    const std::vector<uint64_t> zc = atom_zorder(op);
+    // phase 1: blocks with the same source box (level and first source atom name
+    // it) stack the 8-row groups of their R
+    std::map<std::tuple<int, int, int>, std::vector<int>> groups;
+    for (int i = 0; i < nb; ++i) {
+        const auto& b = op.blocks[i];
+        if (b.rank > 0) groups[{b.level, op.block_atoms[b.s_off], b.ns}].push_back(i);
+    }
+    std::vector<int> grp_t;
+    struct Tile {
+        int rep, grp0, ngrp, run0, nrun;
+        uint64_t key;
+    };
+    std::vector<Tile> tiles;
+    std::vector<WsRun> runs;
+    for (const auto& kv : groups) {
+        const int rep = kv.second.front();
+        const FarBlock& rb = op.blocks[rep];
+        uint64_t zmin = ~0ull;
+        for (int s = 0; s < rb.ns; ++s) zmin = std::min(zmin, zc[op.block_atoms[rb.s_off + s]]);
+        Tile T{rep, (int)grp_t.size(), 0, (int)runs.size(), 0, zmin};
+        auto flush = [&] {
+            if (T.ngrp == 0) return;
+            grp_t.resize((size_t)T.grp0 + 16, 0);  // a tile's groups are 16 places apart
+            tiles.push_back(T);
+            T = Tile{rep, (int)grp_t.size(), 0, (int)runs.size(), 0, zmin};
+        };
+        for (int i : kv.second) {
+            const WsClass& c = cls[cls_of[i]];
+            const int G = (c.rank + 7) / 8;
+            for (int g = 0; g < G;) {
+                const int take = std::min(G - g, 16 - T.ngrp);
+                runs.push_back(WsRun{c.r_unit + g, G, T.ngrp, take, 0});
+                ++T.nrun;
+                for (int e = 0; e < take; ++e) grp_t.push_back(t0[i] + g + e);
+                T.ngrp += take;
+                g += take;
+                if (T.ngrp == 16) flush();
+            }
+        }
+        flush();
+    }
+    upload(op.d_ws_grp, grp_t.empty() ? std::vector<int>{0} : grp_t);
+    // phase 2: per atom the chunks of every (block, slot) touching it
+    std::vector<int> cnt(op.N + 1, 0);
+    for (int i = 0; i < nb; ++i) {
+        const auto& b = op.blocks[i];
+        if (b.rank == 0) continue;
+        for (int s = 0; s < b.nt; ++s) cnt[op.block_atoms[b.t_off + s] + 1] += (b.rank + 7) / 8;
+    }
+    for (int a = 0; a < op.N; ++a) cnt[a + 1] += cnt[a];
+    std::vector<int> fill(cnt.begin(), cnt.end() - 1), qidx(std::max(1, cnt[op.N])), tidx(std::max(1, cnt[op.N]));
+    for (int i = 0; i < nb; ++i) {
+        const auto& b = op.blocks[i];
+        if (b.rank == 0) continue;
+        const WsClass& c = cls[cls_of[i]];
+        const int G = (c.rank + 7) / 8;
+        for (int s = 0; s < b.nt; ++s) {
+            int& f = fill[op.block_atoms[b.t_off + s]];
+            for (int g = 0; g < G; ++g, ++f) {
+                qidx[f] = (int)(c.q_chunk + (int64_t)s * G + g);
+                tidx[f] = t0[i] + g;
+            }
+        }
+    }
+    upload(op.d_ws_kptr, cnt);
+    upload(op.d_ws_qidx, qidx);
+    upload(op.d_ws_tidx, tidx);
+    // items per tile shape, mapped to one CTA per SM
+    for (int v = 0; v < 2; ++v) {
+        const int ks = v ? 16 : 32;
+        std::vector<WsItem1> i1;
+        std::vector<WsRun> rv;
+        std::vector<double> w1;
+        std::vector<uint64_t> k1;
+        for (size_t i = 0; i < tiles.size(); ++i) {
+            const Tile& A = tiles[i];
+            const bool two = v && i + 1 < tiles.size() && tiles[i + 1].rep == A.rep;
+            const Tile* Bt = two ? &tiles[i + 1] : nullptr;
+            i1.push_back(WsItem1{A.rep, op.block_prob.empty() ? 0 : op.block_prob[A.rep], A.grp0, A.run0,
+                                 {A.nrun, two ? Bt->nrun : 0}, {A.ngrp, two ? Bt->ngrp : 0}});
+            w1.push_back(tile_cost(8ll * per * op.blocks[A.rep].ns, ks));
+            k1.push_back(A.key);
+            if (two) ++i;
+        }
+        std::vector<WsItem2> i2;
+        std::vector<double> w2;
+        std::vector<uint64_t> k2;
+        for (int a = 0; a < op.N; ++a)
+            for (int rt = 0; rt < nrt; rt += v + 1) {
+                auto rows = [&](int t) { return std::max(0, std::min(128, op.np - t * 128)); };
+                i2.push_back(WsItem2{a, op.atom_prob.empty() ? 0 : op.atom_prob[a], rt, {rows(rt), v ? rows(rt + 1) : 0}});
+                w2.push_back(tile_cost(8ll * (cnt[a + 1] - cnt[a]), ks));
+                k2.push_back(zc[a]);
+            }
+        auto place = [&](auto& items, const std::vector<double>& w, const std::vector<uint64_t>& key, DevBuf& d_items,
+                         DevBuf& d_cta) {
+            using I = typename std::decay_t<decltype(items)>::value_type;
+            std::vector<int4> dummy(items.size(), make_int4(0, 0, 0, 0)), out;
+            std::vector<int> cta, perm;
+            pack_lpt(dummy, w, n_cta, out, cta, &perm, &key);
+            std::vector<I> sorted(std::max<size_t>(1, items.size()));
+            for (size_t i = 0; i < perm.size(); ++i) sorted[i] = items[perm[i]];
+            upload(d_items, sorted);
+            upload(d_cta, cta);
+        };
+        op.n_ws1[v] = (int)i1.size();
+        place(i1, w1, k1, op.d_ws1_items[v], op.d_ws1_cta[v]);
+        place(i2, w2, k2, op.d_ws2_items[v], op.d_ws2_cta[v]);
+        upload(op.d_ws_runs[v], runs.empty() ? std::vector<WsRun>{WsRun{}} : runs);
+    }
+    op.ws_ready = true;
 }
 
 }  // namespace vie

@@ -60,6 +60,33 @@ def test_apply(array, tol, precision, nrhs):
     ctx.close()
 
 
+# atoms of 6 to 450 unknowns (not whole chunks of 8, one to four row tiles), ragged
+# ranks and column counts, one and two 64-column passes, with and without copies.  A
+# split operand keeps 16 bits: 2^-16 per factor and value, 5e-5 of the norm in all.
+@pytest.mark.parametrize("array,tol,nrhs", [("square 3 1", 1e-4, 8), ("square 8 1", 1e-2, 17), ("spiral 20 2", 1e-4, 9),
+                                            ("graded 5 3", 1e-4, 33), ("square 6 5", 1e-3, 12), ("square 5 3", 1e-5, 65)])
+@pytest.mark.parametrize("variant", ["VAR_TCGEN05_WS_BF16X3", "VAR_TCGEN05_WS2_BF16X3"])
+def test_tensor_core_apply(array, tol, nrhs, variant):
+    import torch
+    from paper_2603_10586_gb300 import vie
+    kind, size, nv = array.split()
+    g = (workloads.square_array(int(size), int(nv)) if kind == "square" else
+         workloads.graded_array(int(size), int(nv), 1) if kind == "graded" else workloads.vogel_gold(int(size), int(nv)))
+    ctx = vie.Context(0)
+    op = vie.Operator(ctx, g)
+    op.compress(tol, vie.C64)
+    op.tune(vie.BF16X3, nrhs, force=getattr(vie, variant))
+    X = torch.from_numpy(workloads.random_complex(op.n, 8, nrhs).T.astype(np.complex64).copy()).cuda()
+    Y = torch.empty_like(X)
+    op.apply(X.data_ptr(), Y.data_ptr(), nrhs, vie.BF16X3, 0)
+    torch.cuda.synchronize()
+    ref = _reference(op, g, X.cpu().numpy().astype(np.complex128), False)
+    err = np.linalg.norm(Y.cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert err.max() < 5e-5
+    op.close()
+    ctx.close()
+
+
 @pytest.mark.parametrize("ns,nv,nrhs", [(1, 1, 1), (2, 3, 1), (3, 4, 5), (7, 2, 11), (16, 3, 9), (12, 4, 33)])
 @pytest.mark.parametrize("precision", ["C64", "C128"])
 def test_precond(ns, nv, nrhs, precision):
