@@ -125,62 +125,48 @@ __global__ void __launch_bounds__(kT) k_gather_df(KrylovArgs a, const double2* _
 
 // partial h[col] = sum_r conj(V[r, col]) w[r], double-float products and
 // per-thread sums, float64 across threads; pass 1 takes w from the float32
-// operator output (exact in double-float) and stores it as basis column j+1
-template <bool kFirst>
-__global__ void __launch_bounds__(kT) k_mdot_df(KrylovArgs a, const float2* __restrict__ Y) {
-    const int i = blockIdx.z, cg = blockIdx.y;
-    if (!a.cycling[i]) return;
-    if (!kFirst && a.reorth && !a.reorth[i]) return;
-    const int j = a.ctr[KR_J];
-    const int ncols = j + 1;
-    if (cg * kCG >= ncols) return;
+// operator output (exact in double-float) and stores it as basis column j+1.
+// Bound by the stream of V (16 bytes per 48 float32 operations).  128 threads and
+// one row at a time keep the registers down to five CTAs per SM, twenty warps with
+// eight 16-byte loads each in flight; NC columns per CTA, fewer for the last
+// ones, so that absent columns cost nothing.
+constexpr int kTD = 128;
+template <bool kFirst, int NC>
+__device__ __forceinline__ void mdot_df_cols(const KrylovArgs& a, const float2* __restrict__ Y, int i, int cg, int j) {
     const Rows R = rows_of(a, a.cols[i]);
     const int64_t n = R.len;
-    const float4* V = reinterpret_cast<const float4*>(R.V);
+    const float4* V = reinterpret_cast<const float4*>(R.V) + (int64_t)cg * kCG * n;
     float4* w = reinterpret_cast<float4*>(R.V) + (int64_t)(j + 1) * n;
     const float2* y = kFirst ? Y + (int64_t)i * a.n + R.lo : nullptr;
     const int64_t rows_per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
-    float4 acc[kCG];
+    float4 acc[NC];
 #pragma unroll
-    for (int c = 0; c < kCG; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = 0; c < NC; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     double wn = 0.0;  // pass 1: ||w||^2 partials (blocks of column group 0)
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += 2 * kT) {
-        const bool second = r + kT < r1;
-        float4 wv, wv2 = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t r = r0 + threadIdx.x; r < r1; r += kTD) {
+        float4 v[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c] = __ldcs(V + c * n + r);
+        float4 wv;
         if (kFirst) {
             const float2 y1 = y[r];
             wv = make_float4(y1.x, y1.y, 0.f, 0.f);
-            if (second) {
-                const float2 y2 = y[r + kT];
-                wv2 = make_float4(y2.x, y2.y, 0.f, 0.f);
-            }
             if (cg == 0) {
                 w[r] = wv;
-                if (second) w[r + kT] = wv2;
-                wn += (double)wv.x * wv.x + (double)wv.y * wv.y + (double)wv2.x * wv2.x + (double)wv2.y * wv2.y;
+                wn += (double)wv.x * wv.x + (double)wv.y * wv.y;
             }
         } else {
             wv = w[r];
-            if (second) wv2 = w[r + kT];
-        }
-        float4 v1[kCG], v2[kCG];
-#pragma unroll
-        for (int c = 0; c < kCG; ++c) {
-            const int col = cg * kCG + c;
-            v1[c] = col < ncols ? V[(int64_t)col * n + r] : make_float4(0.f, 0.f, 0.f, 0.f);
-            v2[c] = (col < ncols && second) ? V[(int64_t)col * n + r + kT] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int c = 0; c < kCG; ++c) {
-            df_cmac_conj(acc[c], v1[c], wv);
-            df_cmac_conj(acc[c], v2[c], wv2);
-        }
+        for (int c = 0; c < NC; ++c) df_cmac_conj(acc[c], v[c], wv);
     }
-    __shared__ double2 sh[kT / 32][kCG];
+    __shared__ double2 sh[kTD / 32][kCG];
+    __shared__ double shn[kTD / 32];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int c = 0; c < kCG; ++c) {
+    for (int c = 0; c < NC; ++c) {
         double re = (double)acc[c].x + (double)acc[c].z, im = (double)acc[c].y + (double)acc[c].w;
         for (int o = 16; o > 0; o >>= 1) {
             re += __shfl_down_sync(0xffffffffu, re, o);
@@ -189,24 +175,39 @@ __global__ void __launch_bounds__(kT) k_mdot_df(KrylovArgs a, const float2* __re
         if (lane == 0) sh[wid][c] = make_double2(re, im);
     }
     // pass 1: the squared norm of w goes to partial slot j + 1 (<= m < hs), beside the dots
-    __shared__ double shn[kT / 32];
     if (kFirst && cg == 0) {
         for (int o = 16; o > 0; o >>= 1) wn += __shfl_down_sync(0xffffffffu, wn, o);
         if (lane == 0) shn[wid] = wn;
     }
     __syncthreads();
-    if (threadIdx.x < kCG) {
-        const int col = cg * kCG + threadIdx.x;
-        if (col < ncols) {
-            double2 s = make_double2(0.0, 0.0);
-            for (int w2 = 0; w2 < kT / 32; ++w2) s += sh[w2][threadIdx.x];
-            a.part[((int64_t)i * a.hs + col) * gridDim.x + blockIdx.x] = s;
-        }
+    const int nc = min(kCG, j + 1 - cg * kCG);
+    if ((int)threadIdx.x < nc) {
+        double2 s = make_double2(0.0, 0.0);
+        for (int w2 = 0; w2 < kTD / 32; ++w2) s += sh[w2][threadIdx.x];
+        a.part[((int64_t)i * a.hs + cg * kCG + threadIdx.x) * gridDim.x + blockIdx.x] = s;
     }
     if (kFirst && cg == 0 && threadIdx.x == 0) {
         double t = 0.0;
-        for (int w2 = 0; w2 < kT / 32; ++w2) t += shn[w2];
-        a.part[((int64_t)i * a.hs + ncols) * gridDim.x + blockIdx.x] = make_double2(t, 0.0);
+        for (int w2 = 0; w2 < kTD / 32; ++w2) t += shn[w2];
+        a.part[((int64_t)i * a.hs + j + 1) * gridDim.x + blockIdx.x] = make_double2(t, 0.0);
+    }
+}
+template <bool kFirst>
+__global__ void __launch_bounds__(kTD, 5) k_mdot_df(KrylovArgs a, const float2* __restrict__ Y) {
+    const int i = blockIdx.z, cg = blockIdx.y;
+    if (!a.cycling[i]) return;
+    if (!kFirst && a.reorth && !a.reorth[i]) return;
+    const int j = a.ctr[KR_J], nc = j + 1 - cg * kCG;
+    if (nc <= 0) return;
+    switch (min(nc, kCG)) {
+        case 1: mdot_df_cols<kFirst, 1>(a, Y, i, cg, j); break;
+        case 2: mdot_df_cols<kFirst, 2>(a, Y, i, cg, j); break;
+        case 3: mdot_df_cols<kFirst, 3>(a, Y, i, cg, j); break;
+        case 4: mdot_df_cols<kFirst, 4>(a, Y, i, cg, j); break;
+        case 5: mdot_df_cols<kFirst, 5>(a, Y, i, cg, j); break;
+        case 6: mdot_df_cols<kFirst, 6>(a, Y, i, cg, j); break;
+        case 7: mdot_df_cols<kFirst, 7>(a, Y, i, cg, j); break;
+        default: mdot_df_cols<kFirst, 8>(a, Y, i, cg, j); break;
     }
 }
 
@@ -229,7 +230,16 @@ __global__ void __launch_bounds__(kT) k_maxpy_df(KrylovArgs a) {
     double nacc = 0.0;
     for (int64_t r = (int64_t)blockIdx.x * kT + threadIdx.x; r < n; r += (int64_t)gridDim.x * kT) {
         float4 acc = w[r];
-        for (int c = 0; c <= j; ++c) df_cmsub(acc, V[(int64_t)c * n + r], hs[c]);
+        const float4* v = V + r;
+        int c = 0;
+        for (; c + 8 <= j + 1; c += 8, v += 8 * n) {  // eight columns in flight; the sums keep their order
+            float4 q[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) q[u] = __ldcs(v + u * n);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) df_cmsub(acc, q[u], hs[c + u]);
+        }
+        for (; c <= j; ++c, v += n) df_cmsub(acc, __ldcs(v), hs[c]);
         acc = df_normed(acc);
         w[r] = acc;
         const double2 d = df_to(acc);
@@ -265,7 +275,8 @@ __global__ void __launch_bounds__(kT) k_xupdate_df(KrylovArgs a, double2* __rest
     float2* d = D ? D + (int64_t)i * a.n + R.lo : nullptr;
     for (int64_t r = (int64_t)blockIdx.x * kT + threadIdx.x; r < n; r += (int64_t)gridDim.x * kT) {
         double2 acc = make_double2(0.0, 0.0);
-        for (int l = 0; l < jd; ++l) cfma(acc, df_to(V[(int64_t)l * n + r]), ys[l]);
+#pragma unroll 8
+        for (int l = 0; l < jd; ++l) cfma(acc, df_to(__ldcs(V + (int64_t)l * n + r)), ys[l]);
         x[r] += acc;
         if (d) d[r] = make_float2((float)acc.x, (float)acc.y);
     }
@@ -396,12 +407,13 @@ __global__ void __launch_bounds__(kT) k_reduce(KrylovArgs a, int nchunk) {
     if (kFirst && sel) {
         if (lane == 0) hn[wid] = hsq;
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (wid == 0) {
             double h2 = 0.0, w2 = 0.0;
             for (int x = 0; x < kT / 32; ++x) h2 += hn[x];
             const double2* p = a.part + ((int64_t)i * a.hs + j + 1) * nchunk;
-            for (int x = 0; x < nchunk; ++x) w2 += p[x].x;
-            a.reorth[i] = (w2 - h2 < 0.5 * w2) || !(w2 > 0.0) || !isfinite(w2 - h2) ? 1 : 0;
+            for (int x = lane; x < nchunk; x += 32) w2 += p[x].x;
+            for (int o = 16; o > 0; o >>= 1) w2 += __shfl_down_sync(0xffffffffu, w2, o);
+            if (lane == 0) a.reorth[i] = (w2 - h2 < 0.5 * w2) || !(w2 > 0.0) || !isfinite(w2 - h2) ? 1 : 0;
         }
     }
 }
@@ -448,7 +460,33 @@ __global__ void __launch_bounds__(kT) k_maxpy(KrylovArgs a) {
     }
 }
 
-// one thread per slot: new Hessenberg column, Givens rotations
+// the earlier rotations on the new Hessenberg column, a CTA per slot: the column
+// and the rotations come to shared memory at once, one thread runs the chain (from
+// global memory, every link waited for its loads: 36 us per step at 32 slots)
+__global__ void __launch_bounds__(64) k_rotate(KrylovArgs a) {
+    const int i = blockIdx.x;
+    if (!a.cycling[i]) return;
+    const int j = a.ctr[KR_J], m = a.m, tid = threadIdx.x;
+    __shared__ double2 h[kMaxRestart + 1], c[kMaxRestart], s[kMaxRestart];
+    double2* Hc = a.H + ((int64_t)i * m + j) * (m + 1);
+    for (int l = tid; l < j; l += 64) {
+        h[l] = Hc[l];
+        c[l] = a.cs[(int64_t)i * m + l];
+        s[l] = a.sn[(int64_t)i * m + l];
+    }
+    if (tid == 0) h[j] = Hc[j];
+    __syncthreads();
+    if (tid == 0)
+        for (int l = 0; l < j; ++l) {
+            const double2 x = h[l], y = h[l + 1];
+            h[l] = cmulc(c[l], x) + cmulc(s[l], y);
+            h[l + 1] = cmul(c[l], y) - cmul(s[l], x);
+        }
+    __syncthreads();
+    for (int l = tid; l <= j; l += 64) Hc[l] = h[l];
+}
+
+// one thread per slot: the rotated Hessenberg column's own Givens rotation
 // G = [[conj c, conj s], [-s, c]], residual estimate |g_{j+1}| / ||M^-1 b||
 __global__ void k_givens(KrylovArgs a, int k, int nblk, cudaGraphConditionalHandle hnd, int use_handle) {
     const int i = threadIdx.x;
@@ -464,11 +502,6 @@ __global__ void k_givens(KrylovArgs a, int k, int nblk, cudaGraphConditionalHand
         double2* sn = a.sn + (int64_t)i * m;
         double2* g = a.g + (int64_t)i * (m + 1);
         Hc[j + 1] = make_double2(hn, 0.0);
-        for (int l = 0; l < j; ++l) {
-            const double2 x = Hc[l], y = Hc[l + 1];
-            Hc[l] = cmulc(cs[l], x) + cmulc(sn[l], y);
-            Hc[l + 1] = cmul(cs[l], y) - cmul(sn[l], x);
-        }
         const double2 x = Hc[j], y = Hc[j + 1];
         const double den = sqrt(x.x * x.x + x.y * x.y + y.x * y.x + y.y * y.y);
         const double2 cj = den > 0.0 ? (1.0 / den) * x : make_double2(1.0, 0.0);
@@ -661,7 +694,8 @@ int kr_nblk(int64_t n, int k, int n_sm) {
 
 int kr_nchunk(int64_t n, int k, int m, int n_sm) {
     const int groups = std::max(1, std::min(4, (m + kCG - 1) / kCG));  // column groups live on average
-    const int64_t want = ((int64_t)n_sm * 8 + (int64_t)k * groups - 1) / ((int64_t)k * groups);
+    // ~20 CTAs of the projections per SM in total, with at least 1,024 rows each
+    const int64_t want = ((int64_t)n_sm * 20 + (int64_t)k * groups - 1) / ((int64_t)k * groups);
     const int64_t cap = (n + 4 * kT - 1) / (4 * kT);
     return (int)std::max<int64_t>(1, std::min(want, cap));
 }
@@ -688,7 +722,7 @@ void kr_project(const KrylovArgs& a, const void* Y, bool c64, int pass, int k, i
     const int ncg = (a.m + kCG - 1) / kCG;
     dim3 gd(nchunk, ncg, k);
     if (pass == 1) {
-        if (a.df) k_mdot_df<true><<<gd, kT, 0, s>>>(a, static_cast<const float2*>(Y));
+        if (a.df) k_mdot_df<true><<<gd, kTD, 0, s>>>(a, static_cast<const float2*>(Y));
         else if (c64) k_mdot<float2, true><<<gd, kT, 0, s>>>(a, static_cast<const float2*>(Y));
         else k_mdot<double2, true><<<gd, kT, 0, s>>>(a, static_cast<const double2*>(Y));
         VIE_CHECK_LAUNCH();
@@ -698,7 +732,7 @@ void kr_project(const KrylovArgs& a, const void* Y, bool c64, int pass, int k, i
         else k_maxpy<false><<<dim3(nblk, k), kT, 0, s>>>(a);
         VIE_CHECK_LAUNCH();
     } else {
-        if (a.df) k_mdot_df<false><<<gd, kT, 0, s>>>(a, nullptr);  // returns at once where pass 2 is not needed
+        if (a.df) k_mdot_df<false><<<gd, kTD, 0, s>>>(a, nullptr);  // returns at once where pass 2 is not needed
         else k_mdot<double2, false><<<gd, kT, 0, s>>>(a, nullptr);
         VIE_CHECK_LAUNCH();
         k_reduce<false><<<k, kT, 0, s>>>(a, nchunk);
@@ -713,6 +747,8 @@ void kr_project(const KrylovArgs& a, const void* Y, bool c64, int pass, int k, i
 
 void kr_givens(const KrylovArgs& a, int k, int nblk, cudaGraphConditionalHandle hnd, int use_handle, cudaStream_t s) {
     if (k > 1024) fail(VIE_ERR_INVALID_ARG, "more than 1024 right-hand sides in one solve");
+    k_rotate<<<k, 64, 0, s>>>(a);
+    VIE_CHECK_LAUNCH();
     k_givens<<<1, slot_threads(k), 0, s>>>(a, k, nblk, hnd, use_handle);
     VIE_CHECK_LAUNCH();
 }
