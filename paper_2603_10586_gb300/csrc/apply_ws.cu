@@ -114,15 +114,15 @@ struct WsGeom {
     // accumulator buffers: each holds MT accumulators of 4 nmax columns
     __host__ __device__ static constexpr int nbuf(int nmax) { return kWsTmemCols / (MT * 4 * nmax) >= 2 ? 2 : 1; }
 };
-static_assert(WsGeom<1>::stages(64) == 3 && WsGeom<1>::stages(16) == 5, "ring sizes");
+static_assert(WsGeom<1>::stages(32) == 4 && WsGeom<1>::stages(16) == 5, "ring sizes");
 static_assert(WsGeom<2>::stages(64) == 4 && WsGeom<2>::stages(16) == 6, "ring sizes");
 static_assert(WsGeom<2>::stride(16) % 1024 == 0 && WsGeom<1>::stride(16) % 1024 == 0, "stage alignment");
 
 // The ring: ns stages of `stride` bytes.  A stage holds the A planes, then the
 // two B stacks; chunk (slot, row, q) of a stack sits at q (4 nmma) + slot nmma
 // + row.  nmax, the widest tile's column count rounded up to 16, sets the
-// stride, and the stage count is what fits: for MT = 1, 5 stages up to 16
-// right-hand sides, 4 up to 48, 3 up to 64; for MT = 2, 6, 5 and 4.
+// stride, and the stage count is what fits: for MT = 1 (up to 32 columns), 5
+// stages up to 16 right-hand sides, else 4; for MT = 2, 6 up to 16, 5 up to 48, 4 up to 64.
 struct WsRing {
     unsigned char* base;
     uint32_t stride, bstack;  // bytes per stage; chunks per B stack
@@ -487,7 +487,7 @@ __device__ void ws_teardown(WsCtl& ctl, uint32_t ns, int* err) {
 // The B operand of a tile's stages st, st + groups, ...: a thread's NS segments of
 // 8 values (neighbouring threads take neighbouring columns of one K chunk, so
 // their 16-byte stores fill whole shared-memory wavefronts), read one stage
-// ahead (NS <= 2) and before the wait for the slot, then split and stored.
+// ahead and before the wait for the slot, then split and stored.
 // Returns the first stage not done, -1 on an abort.
 struct ProduceArgs {
     int gtid, groups;
@@ -497,7 +497,6 @@ template <int MT, int NS, class TileT>
 __device__ __forceinline__ int ws_produce(WsCtl& ctl, const WsRing& ring, const TileT& T, RingPos& p,
                                           const ProduceArgs& a, int st) {
     using G = WsGeom<MT>;
-    constexpr bool kAhead = NS <= 2;
     const int nm = T.nmma, nseg = nm * G::KQ, lane = threadIdx.x & 31;
     int col[NS], kq[NS];
     typename TileT::At at[NS];
@@ -517,16 +516,13 @@ __device__ __forceinline__ int ws_produce(WsCtl& ctl, const WsRing& ring, const 
                 T.advance(at[u], a.groups * G::KS);
             }
     };
-    if (kAhead) load(st);
+    load(st);
     for (; st < T.nst; st += a.groups) {
-        Chunks cur[kAhead ? NS : 1];
-        if (!kAhead) load(st);
-        if (kAhead) {
+        Chunks cur[NS];
 #pragma unroll
-            for (int u = 0; u < NS; ++u)
-                if (col[u] >= 0) cur[kAhead ? u : 0] = split8(vb[u]);
-            if (st + a.groups < T.nst) load(st + a.groups);
-        }
+        for (int u = 0; u < NS; ++u)
+            if (col[u] >= 0) cur[u] = split8(vb[u]);
+        if (st + a.groups < T.nst) load(st + a.groups);
         int ok = 1;
         if (lane == 0) ok = ws_wait(ctl, ctl.empty[p.slot], p.par ^ 1, a.lim);
         if (!__shfl_sync(0xffffffffu, ok, 0)) return -1;
@@ -534,7 +530,7 @@ __device__ __forceinline__ int ws_produce(WsCtl& ctl, const WsRing& ring, const 
         uint4* b1 = ring.b(p.slot, 1);
 #pragma unroll
         for (int u = 0; u < NS; ++u)
-            if (col[u] >= 0) put8_ws(b0, b1, nm, col[u], kq[u], kAhead ? cur[kAhead ? u : 0] : split8(vb[u]));
+            if (col[u] >= 0) put8_ws(b0, b1, nm, col[u], kq[u], cur[u]);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctl.full_b[p.slot]));
@@ -603,9 +599,8 @@ __device__ void ws_run(WsCtl& ctl, const WsRing& ring, int nmax, long long lim, 
             }
             const int nseg = T.nmma * G::KQ;  // segments of 8 values, 64 threads
             const ProduceArgs pa{gtid, (int)ngroups, lim};
-            const int st = nseg <= 64    ? ws_produce<MT, 1>(ctl, ring, T, p, pa, wait)
-                           : nseg <= 128 ? ws_produce<MT, 2>(ctl, ring, T, p, pa, wait)
-                                         : ws_produce<MT, 4>(ctl, ring, T, p, pa, wait);
+            const int st = nseg <= 64 ? ws_produce<MT, 1>(ctl, ring, T, p, pa, wait)
+                                      : ws_produce<MT, 2>(ctl, ring, T, p, pa, wait);
             if (st < 0) return false;
             wait = st - T.nst;
             return true;
@@ -898,7 +893,10 @@ static void apply_far_ws(Op& op, const float2* x, int64_t ldx, float2* F, int64_
 }
 
 void apply_far_umma_ws(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s) {
-    apply_far_ws<1>(op, x, ldx, F, ldf, nrhs, s);
+    // wider, a producer thread would hold four segments of B of one 32-K stage: two
+    // row tiles per B tile take half of them
+    if (nrhs <= 32) apply_far_ws<1>(op, x, ldx, F, ldf, nrhs, s);
+    else apply_far_ws<2>(op, x, ldx, F, ldf, nrhs, s);
 }
 
 void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, cudaStream_t s) {
