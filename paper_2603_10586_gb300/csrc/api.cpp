@@ -152,6 +152,7 @@ vie_ctx* ctx_of(vie_op* op) { return op ? static_cast<vie_ctx*>(op->o.ctx->owner
 // admitted with; the peak shows what the request really held
 void ctx_set_cap(vie_ctx* ctx, int64_t cap) {
     ctx->c.cap = cap;
+    ctx->c.admitted = cap > 0;
     ctx->c.peak = ctx->c.allocated.load();
 }
 int64_t ctx_peak(vie_ctx* ctx) { return ctx->c.peak.load(); }
@@ -195,6 +196,18 @@ int vie_create(vie_ctx** out, const vie_ctx_opts* opts) {
         VIE_CUDA(cudaGetDeviceProperties(&prop, c.device));
         c.n_sm = prop.multiProcessorCount;
         VIE_CUDA(cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking));
+        cudaMemPoolProps pp = {};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.handleTypes = cudaMemHandleTypeNone;
+        pp.location.type = cudaMemLocationTypeDevice;
+        pp.location.id = c.device;
+        if (cudaMemPoolCreate(&c.pool, &pp) == cudaSuccess) {
+            uint64_t keep = Ctx::kPoolKeep;
+            cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        } else {  // ordinary allocations instead
+            c.pool = nullptr;
+            cudaGetLastError();
+        }
         VIE_BLAS(cublasCreate(&c.blas));
         VIE_BLAS(cublasSetStream(c.blas, c.stream));
         size_t fr = 0, tot = 0;
@@ -216,6 +229,11 @@ int vie_create(vie_ctx** out, const vie_ctx_opts* opts) {
 static void free_ctx(vie_ctx* ctx) {
     cudaSetDevice(ctx->c.device);
     if (ctx->c.blas) cublasDestroy(ctx->c.blas);
+    if (ctx->c.pool) {
+        ctx->c.unions.clear();  // (their buffers are not pooled; freed before the stream)
+        cudaStreamSynchronize(ctx->c.stream);
+        cudaMemPoolDestroy(ctx->c.pool);
+    }
     if (ctx->c.stream) cudaStreamDestroy(ctx->c.stream);
     delete ctx;
 }
@@ -321,6 +339,7 @@ int vie_assemble(vie_ctx* ctx, const vie_geometry* g, double wavelength, vie_op*
             o.type_atom_off[t + 1] = (int)flat.size();
         }
         upload(o.d_atoms_by_type, flat);
+        TmpScope tmp(ctx->c.stream);
         // grid hierarchy and far-block lists
         build_tree(o);
         // self blocks, their inverses (float64) and float32 copies

@@ -463,7 +463,7 @@ bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
         if (op.d_part.bytes < np) op.d_part.alloc(np);
         if (op.d_ct.bytes < nt) op.d_ct.alloc(nt);
     } catch (const Error& e) {
-        if (e.status != VIE_ERR_OOM) throw;
+        if (e.status != VIE_ERR_OOM || op.ctx->admitted) throw;
         return false;
     }
     return true;

@@ -705,11 +705,11 @@ void assemble_self_blocks(Op& op) {
     const DevMesh& m = op.dmesh;
     const int np = m.np;
     size_t stride = table_stride(m);
-    DevBuf tab(stride * sizeof(double2));
+    TmpBuf tab(stride * sizeof(double2));
     const int w1o = 2 * m.nv - 1;
-    DevBuf otab((size_t)13 * w1o * w1o * w1o * sizeof(double2));  // voxel/voxel integrals per offset
+    TmpBuf otab((size_t)13 * w1o * w1o * w1o * sizeof(double2));  // voxel/voxel integrals per offset
     op.d_zself64.alloc((size_t)op.T * np * np * sizeof(double2));
-    DevBuf jobs(sizeof(PairJob)), dst(sizeof(void*)), ldb(sizeof(int64_t));
+    TmpBuf jobs(sizeof(PairJob)), dst(sizeof(void*)), ldb(sizeof(int64_t));
     cudaStream_t s = op.ctx->stream;
     for (int t = 0; t < op.T; ++t) {
         double h = op.h[t];
@@ -771,11 +771,12 @@ void assemble_pairs_as(Op& op, const PairJob* d_jobs, int n_jobs, void* const* d
     size_t per_job = stride * sizeof(T2);
     int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_jobs, ((size_t)2 << 30) / per_job));
     chunk = std::min(chunk, 65535);  // jobs run along grid y / z
-    DevBuf tab((size_t)chunk * per_job);
+    TmpScope scope(s);
+    TmpBuf tab((size_t)chunk * per_job);
     const T tol = T(2.0 / op.wavelength);
     const int nv2 = m.nvox * m.nvox;
     const int ns = std::max(m.nvox, m.nsurf) * m.nsurf;
-    DevBuf npart;
+    TmpBuf npart;
     if (norm_out)
         npart.alloc((size_t)chunk * ((m.np + kEntRows - 1) / kEntRows) * ((m.np + kEntCols - 1) / kEntCols) *
                     sizeof(double));

@@ -66,16 +66,20 @@ struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
     Ctx* owner = nullptr;
+    bool tmp = false;               // a TmpBuf
+    cudaStream_t stream = nullptr;  // pooled memory: the stream it belongs to
     DevBuf() = default;
     explicit DevBuf(size_t b) { alloc(b); }
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
-    DevBuf(DevBuf&& o) noexcept : p(o.p), bytes(o.bytes), owner(o.owner) { o.p = nullptr; o.bytes = 0; o.owner = nullptr; }
+    DevBuf(DevBuf&& o) noexcept : p(o.p), bytes(o.bytes), owner(o.owner), tmp(o.tmp), stream(o.stream) {
+        o.p = nullptr; o.bytes = 0; o.owner = nullptr; o.stream = nullptr;
+    }
     DevBuf& operator=(DevBuf&& o) noexcept {
         if (this != &o) {
             release();
-            p = o.p; bytes = o.bytes; owner = o.owner;
-            o.p = nullptr; o.bytes = 0; o.owner = nullptr;
+            p = o.p; bytes = o.bytes; owner = o.owner; tmp = o.tmp; stream = o.stream;
+            o.p = nullptr; o.bytes = 0; o.owner = nullptr; o.stream = nullptr;
         }
         return *this;
     }
@@ -85,10 +89,34 @@ struct DevBuf {
     template <class T> T* as() const { return static_cast<T*>(p); }
 };
 
+// A buffer of one call whose every use is on the stream of the enclosing
+// TmpScope.  Up to kPoolMax bytes it comes from the context's stream-ordered
+// pool: cudaMalloc and cudaFree cost ~15 and ~20 us and a device-wide wait each,
+// and a small request made 180 of them, half of its 18 ms.  Larger ones, and those
+// outside a scope, are ordinary allocations.
+struct TmpBuf : DevBuf {
+    static constexpr size_t kPoolMax = (size_t)64 << 20;
+    TmpBuf() { tmp = true; }
+    explicit TmpBuf(size_t b) { tmp = true; alloc(b); }
+    TmpBuf(TmpBuf&&) = default;
+    TmpBuf& operator=(TmpBuf&&) = default;
+};
+// makes TmpBufs of this thread belong to stream `s` (restored on exit)
+struct TmpScope {
+    cudaStream_t prev;
+    bool prev_on;
+    explicit TmpScope(cudaStream_t s);
+    ~TmpScope();
+};
+
 template <class T>
 void upload(DevBuf& d, const std::vector<T>& h) {
     d.alloc(std::max<size_t>(1, h.size() * sizeof(T)));
-    if (!h.empty()) VIE_CUDA(cudaMemcpy(d.p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
+    if (h.empty()) return;
+    if (d.stream)  // pooled: in stream order (a pageable source has been read on return)
+        VIE_CUDA(cudaMemcpyAsync(d.p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, d.stream));
+    else
+        VIE_CUDA(cudaMemcpy(d.p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
 }
 
 // ---------------------------------------------------------------------------
@@ -249,6 +277,8 @@ struct Ctx {
     int device = 0;
     int n_sm = 0;
     cudaStream_t stream = nullptr;
+    cudaMemPool_t pool = nullptr;  // TmpBufs; keeps at most kPoolKeep bytes between calls
+    static constexpr size_t kPoolKeep = (size_t)256 << 20;
     cublasHandle_t blas = nullptr;
     std::string err;
     size_t budget = 0;
@@ -259,6 +289,7 @@ struct Ctx {
     // (0: none) above which an allocation is refused with VIE_ERR_OOM
     std::atomic<int64_t> allocated{0}, peak{0};
     std::atomic<int64_t> cap{0};
+    bool admitted = false;  // a server's slot: a request that meets the cap is run again with more
     // joined operators of recent vie_solve_batch calls (block-diagonal unions of
     // their problems), reused while the same operators with the same factors
     // come again; declared last so that they are freed first
@@ -440,7 +471,9 @@ void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t
 // apply_tile.cu: far apply by register tiles over classes of blocks that share
 // their factors.  tile_reserve: its scratch for nrhs columns of `elem`-byte
 // vector elements; false when the memory is not there (or would have to be allocated
-// while `s` is capturing), and the per-block kernels run instead.
+// while `s` is capturing), and the per-block kernels run instead.  In a server's slot
+// VIE_ERR_OOM: the request runs again with a larger footprint, and its result does not
+// depend on the cap it first met.
 bool tile_pays(const Op& op, int nrhs);
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s);
 template <class TF, class TX, class TO>

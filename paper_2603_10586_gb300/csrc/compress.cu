@@ -337,13 +337,22 @@ __global__ void k_trmul(const T2* Y, int m, int64_t ystride, const T2* Minv, con
     }
 }
 
-// dst = conj(src)
+// factor pieces into the factor store, one job per blockIdx.y: dst = src, or
+// conj(src) for the mirror of a compressed block
 template <class T2>
-__global__ void k_conj_copy(const T2* src, T2* dst, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T2 v = src[i];
-        v.y = -v.y;
-        dst[i] = v;
+struct StoreJob {
+    const T2* src;
+    long long dst, len;
+    int conj;
+};
+template <class T2>
+__global__ void k_store(const StoreJob<T2>* __restrict__ jobs, T2* __restrict__ out) {
+    const StoreJob<T2> j = jobs[blockIdx.y];
+    T2* d = out + j.dst;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < j.len; i += (int64_t)gridDim.x * blockDim.x) {
+        T2 v = j.src[i];
+        if (j.conj) v.y = -v.y;
+        d[i] = v;
     }
 }
 
@@ -549,7 +558,7 @@ struct Compressor {
     double tol;
     cudaStream_t s;
     cublasHandle_t h;
-    std::vector<DevBuf> stores;          // staging factor stores (one per batch)
+    std::vector<TmpBuf> stores;          // staging factor stores (one per batch)
     std::vector<std::pair<int, int64_t>> where;  // per block: (store, offset of Q); R^H follows Q
     std::map<std::tuple<int, int, int>, int> class_rank;  // (level, offsets) -> largest rank seen
     uint64_t seed = 0x5eed0001ull;
@@ -646,11 +655,11 @@ struct Compressor {
             const size_t ubytes = ujobs.size() * (size_t)np * np * sizeof(T2);
             // worth it when pairs repeat, and when the distinct blocks fit a modest scratch
             if (ujobs.size() * 2 <= jobs.size() && ubytes <= ((size_t)16 << 30)) {
-                DevBuf ublk(ubytes), unorm(ujobs.size() * sizeof(double));
+                TmpBuf ublk(ubytes), unorm(ujobs.size() * sizeof(double));
                 std::vector<void*> udst(ujobs.size());
                 std::vector<int64_t> uld(ujobs.size(), np);
                 for (size_t u = 0; u < ujobs.size(); ++u) udst[u] = ublk.as<T2>() + u * (size_t)np * np;
-                DevBuf dj, dd, dl, dp, dq;
+                TmpBuf dj, dd, dl, dp, dq;
                 upload(dj, ujobs);
                 upload(dd, udst);
                 upload(dl, uld);
@@ -672,7 +681,7 @@ struct Compressor {
                 return planes;
             }
         }
-        DevBuf dj, dd, dl;
+        TmpBuf dj, dd, dl;
         upload(dj, jobs);
         upload(dd, dst);
         upload(dl, ld);
@@ -696,7 +705,7 @@ struct Compressor {
             total += (int64_t)rank[q] * (m + n);
             total = (total + 31) / 32 * 32;
         }
-        DevBuf store((size_t)std::max<int64_t>(total, 32) * sizeof(T2));
+        TmpBuf store((size_t)std::max<int64_t>(total, 32) * sizeof(T2));
         std::vector<long long> so, dof;  // Q columns then R^H columns
         std::vector<long long> so2, dof2;
         int64_t off = 0;
@@ -720,7 +729,7 @@ struct Compressor {
             cr = std::max(cr, rank[q]);
         }
         if (!so.empty()) {
-            DevBuf a1, a2, a3, a4;
+            TmpBuf a1, a2, a3, a4;
             upload(a1, so);
             upload(a2, dof);
             upload(a3, so2);
@@ -758,7 +767,7 @@ struct Compressor {
                            !(sp && sp[0] == '0');
         bool in_planes = false;
         // 1. form the blocks (col-major m x n, ld = m) and their squared norms
-        DevBuf A((size_t)nb * mn * sizeof(T2)), jobnorm;
+        TmpBuf A((size_t)nb * mn * sizeof(T2)), jobnorm;
         {
             std::vector<PairJob> jobs;
             std::vector<void*> dst(nb);
@@ -776,7 +785,7 @@ struct Compressor {
         }
         double t1 = mark();
         tim[0] += t1 - t0;
-        DevBuf part, normA((size_t)nb * sizeof(double)), est((size_t)nb * sizeof(double));
+        TmpBuf part, normA((size_t)nb * sizeof(double)), est((size_t)nb * sizeof(double));
         // ||A||_F^2 of each block: the sum over its (contiguous) atom-pair jobs
         k_reduce_rows<<<(nb + 127) / 128, 128, 0, s>>>(jobnorm.as<double>(), b0.nt * b0.ns, nb, normA.as<double>());
         VIE_CHECK_LAUNCH();
@@ -784,7 +793,7 @@ struct Compressor {
         VIE_CUDA(cudaMemcpyAsync(hnorm.data(), normA.p, nb * sizeof(double), cudaMemcpyDeviceToHost, s));
         if (cross) {
             // 2'. cross approximation with full pivoting: Q = U, R^H = conj(V)
-            DevBuf U((size_t)nb * m * rcap_pad * sizeof(T2)), VH((size_t)nb * n * rcap_pad * sizeof(T2));
+            TmpBuf U((size_t)nb * m * rcap_pad * sizeof(T2)), VH((size_t)nb * n * rcap_pad * sizeof(T2));
             std::vector<int> rk;
             const CrossStats cs = cross_full_batch<T2>(A.as<T2>(), nb, m, n, normA.as<double>(), tol, rcap, rfull,
                                                        U.as<T2>(), (int64_t)m * rcap_pad, VH.as<T2>(),
@@ -831,14 +840,14 @@ struct Compressor {
         }
 
         // 2. adaptive range finder
-        DevBuf Q((size_t)nb * m * rcap_pad * sizeof(T2));
+        TmpBuf Q((size_t)nb * m * rcap_pad * sizeof(T2));
         VIE_CUDA(cudaMemsetAsync(Q.p, 0, Q.bytes, s));
-        DevBuf alive((size_t)nb * rcap_pad);
+        TmpBuf alive((size_t)nb * rcap_pad);
         VIE_CUDA(cudaMemsetAsync(alive.p, 1, alive.bytes, s));
-        DevBuf Cb((size_t)nb * rcap_pad * kChunk * sizeof(T2));
-        DevBuf gpart, G((size_t)nb * kChunk * kChunk * sizeof(double2)), Minv((size_t)nb * kChunk * kChunk * sizeof(T2));
-        DevBuf d_active(nb * sizeof(int)), d_rbase(nb * sizeof(int));
-        DevBuf pbuf1((size_t)3 * nb * sizeof(void*)), pbuf2((size_t)3 * nb * sizeof(void*)), Cpan;
+        TmpBuf Cb((size_t)nb * rcap_pad * kChunk * sizeof(T2));
+        TmpBuf gpart, G((size_t)nb * kChunk * kChunk * sizeof(double2)), Minv((size_t)nb * kChunk * kChunk * sizeof(T2));
+        TmpBuf d_active(nb * sizeof(int)), d_rbase(nb * sizeof(int));
+        TmpBuf pbuf1((size_t)3 * nb * sizeof(void*)), pbuf2((size_t)3 * nb * sizeof(void*)), Cpan;
         std::vector<int> r(nb, 0), conv(nb, 0);
         // first sketch: the rank prior of this block class (one pass over A), then
         // 32-column passes for the blocks that still need more
@@ -872,13 +881,13 @@ struct Compressor {
                 for (int q = 0; q < nb; ++q) conv[q] = 1;
                 break;
             }
-            DevBuf Y((size_t)nb * m * scols * sizeof(T2));
+            TmpBuf Y((size_t)nb * m * scols * sizeof(T2));
             const uint64_t sseed = seed + 7919ull * step;
             ++step;
             const T2 one = mk(T(1), T(0)), zero = mk(T(0), T(0)), mone = mk(T(-1), T(0));
             if (split) {
                 // [Re Y | Im Y] = A (m x 4n planes) B (4n x 2 scols), then joined
-                DevBuf Wb((size_t)8 * n * scols * sizeof(bf16)), Yf((size_t)nb * m * 2 * scols * sizeof(float));
+                TmpBuf Wb((size_t)8 * n * scols * sizeof(bf16)), Yf((size_t)nb * m * 2 * scols * sizeof(float));
                 k_gauss_bf16<<<(unsigned)(((int64_t)n * scols + 255) / 256), 256, 0, s>>>(Wb.as<bf16>(), n, scols,
                                                                                           sseed);
                 VIE_CHECK_LAUNCH();
@@ -897,7 +906,7 @@ struct Compressor {
                         pb.push_back(Wb.p);
                         pc.push_back(Yf.as<float>() + (size_t)q * fs);
                     }
-                    DevBuf da, db, dc;
+                    TmpBuf da, db, dc;
                     upload(da, pa);
                     upload(db, pb);
                     upload(dc, pc);
@@ -908,7 +917,7 @@ struct Compressor {
                                                  (int)list.size(), CUBLAS_COMPUTE_32F, CUBLAS_GEMM_DEFAULT));
                     VIE_CUDA(cudaStreamSynchronize(s));
                 }
-                DevBuf dl;
+                TmpBuf dl;
                 upload(dl, list);
                 k_join_planes<<<dim3((unsigned)std::min<int64_t>(1024, ((int64_t)m * scols + 255) / 256),
                                      (unsigned)list.size()),
@@ -917,7 +926,7 @@ struct Compressor {
                 VIE_CHECK_LAUNCH();
                 VIE_CUDA(cudaStreamSynchronize(s));  // Wb, Yf go out of scope
             } else {
-              DevBuf W((size_t)n * scols * sizeof(T2));
+              TmpBuf W((size_t)n * scols * sizeof(T2));
               k_gauss<T2><<<(unsigned)(((int64_t)n * scols + 255) / 256), 256, 0, s>>>(W.as<T2>(),
                                                                                        (int64_t)n * scols, sseed);
               VIE_CHECK_LAUNCH();
@@ -933,7 +942,7 @@ struct Compressor {
                         pb.push_back(W.as<T2>());
                         pc.push_back(Y.as<T2>() + (size_t)q * m * scols);
                     }
-                DevBuf da, db, dc;
+                TmpBuf da, db, dc;
                 upload(da, pa);
                 upload(db, pb);
                 upload(dc, pc);
@@ -1052,13 +1061,13 @@ struct Compressor {
         int rmax = *std::max_element(r.begin(), r.end());
         std::vector<unsigned char> halive((size_t)nb * rcap_pad);
         VIE_CUDA(cudaMemcpyAsync(halive.data(), alive.p, halive.size(), cudaMemcpyDeviceToHost, s));
-        DevBuf RH((size_t)nb * n * std::max(rmax, 1) * sizeof(T2));
+        TmpBuf RH((size_t)nb * n * std::max(rmax, 1) * sizeof(T2));
         if (rmax > 0 && split) {
             // [Re R^H | Im R^H] = A^T Bh + A_hi^T Bl (A read as 4m x n), joined per block
             const float2* Qf = reinterpret_cast<const float2*>(Q.p);
             float2* RHf = reinterpret_cast<float2*>(RH.p);
             if (mn >= ((int64_t)1 << 22)) {
-                DevBuf Bh((size_t)8 * m * rmax * sizeof(bf16)), Bl((size_t)4 * m * rmax * sizeof(bf16)),
+                TmpBuf Bh((size_t)8 * m * rmax * sizeof(bf16)), Bl((size_t)4 * m * rmax * sizeof(bf16)),
                     F((size_t)2 * n * rmax * sizeof(float));
                 for (int q = 0; q < nb; ++q) {
                     if (r[q] <= 0) continue;
@@ -1077,7 +1086,7 @@ struct Compressor {
                 VIE_CUDA(cudaStreamSynchronize(s));
             } else {
                 const long long hs = 8LL * m * rmax, ls = 4LL * m * rmax, fs = 2LL * n * rmax;
-                DevBuf Bh((size_t)nb * hs * sizeof(bf16)), Bl((size_t)nb * ls * sizeof(bf16)),
+                TmpBuf Bh((size_t)nb * hs * sizeof(bf16)), Bl((size_t)nb * ls * sizeof(bf16)),
                     F((size_t)nb * fs * sizeof(float));
                 k_split_q<<<dim3((unsigned)std::min<int64_t>(1024, ((int64_t)m * rmax + 255) / 256), nb), 256, 0,
                             s>>>(Qf, m, rmax, (int64_t)m * rcap_pad, Bh.as<bf16>(), hs, Bl.as<bf16>(), ls);
@@ -1240,6 +1249,7 @@ struct Compressor {
             total = (total + 31) / 32 * 32;
         }
         op.d_factors.alloc((size_t)std::max<int64_t>(total, 32) * sizeof(T2));
+        std::vector<StoreJob<T2>> store;
         for (size_t i = 0; i < op.blocks.size(); ++i) {
             auto& b = op.blocks[i];
             if (canon[i] != (int)i) {
@@ -1257,18 +1267,26 @@ struct Compressor {
             if (b.rank == 0) continue;
             if (!b.derived) {
                 const T2* src = stores[where[i].first].template as<T2>() + where[i].second;
-                VIE_CUDA(cudaMemcpyAsync(op.d_factors.as<T2>() + b.q_off, src,
-                                         (size_t)b.rank * (b.m + b.n) * sizeof(T2), cudaMemcpyDeviceToDevice, s));
+                store.push_back({src, b.q_off, (int64_t)b.rank * (b.m + b.n), 0});
             } else {
                 // mirror of block p (A' = A_p^T): Q' = conj(R_p^H), R'^H = conj(Q_p)
                 const int pi = canon[b.mirror];
                 const FarBlock& p = op.blocks[pi];
                 const T2* src = stores[where[pi].first].template as<T2>() + where[pi].second;
                 const int64_t nq = (int64_t)p.rank * p.m, nr = (int64_t)p.rank * p.n;
-                k_conj_copy<T2><<<(unsigned)std::min<int64_t>(4096, (nr + 255) / 256), 256, 0, s>>>(
-                    src + nq, op.d_factors.as<T2>() + b.q_off, nr);
-                k_conj_copy<T2><<<(unsigned)std::min<int64_t>(4096, (nq + 255) / 256), 256, 0, s>>>(
-                    src, op.d_factors.as<T2>() + b.rh_off, nq);
+                store.push_back({src + nq, b.q_off, nr, 1});
+                store.push_back({src, b.rh_off, nq, 1});
+            }
+        }
+        if (!store.empty()) {  // one launch: a copy per block cost ~130 launches on a small array
+            TmpBuf jobs;
+            upload(jobs, store);
+            long long most = 0;
+            for (const auto& j : store) most = std::max(most, j.len);
+            for (size_t j0 = 0; j0 < store.size(); j0 += 65535) {
+                const unsigned cnt = (unsigned)std::min<size_t>(65535, store.size() - j0);
+                k_store<T2><<<dim3((unsigned)std::min<int64_t>(256, (most + 1023) / 1024), cnt), 256, 0, s>>>(
+                    jobs.as<StoreJob<T2>>() + j0, op.d_factors.as<T2>());
                 VIE_CHECK_LAUNCH();
             }
         }
@@ -1281,6 +1299,7 @@ struct Compressor {
 
 void compress_operator(Op& op, double tol, int prec, int method) {
     VIE_BLAS(cublasSetStream(op.ctx->blas, op.ctx->stream));
+    TmpScope tmp(op.ctx->stream);
     // float32-accurate GEMMs on the bf16 tensor cores (BF16x9), float64-accurate
     // fixed-point emulation for the c128 path, where cuBLAS finds them faster
     // (VIE_GEMM_EMULATION=0 keeps plain float32/float64 arithmetic)

@@ -263,7 +263,7 @@ CrossStats cross_full_batch(T2* E, int nb, int m, int n, const double* d_anorm2,
     const int64_t ntile64 = (int64_t)tiles_m * ((n + kXCols - 1) / kXCols);
     if (ntile64 > INT_MAX / 2 || rcap > std::min(m, n)) fail(VIE_ERR_INVALID_ARG, "cross approximation: block too large");
     const int ntile = (int)ntile64;
-    DevBuf d_rank(nb * sizeof(int)), d_piv(nb * sizeof(int2)), d_list(2 * (size_t)nb * sizeof(int)),
+    TmpBuf d_rank(nb * sizeof(int)), d_piv(nb * sizeof(int2)), d_list(2 * (size_t)nb * sizeof(int)),
         d_cnt(4 * sizeof(int)), d_passes(sizeof(unsigned long long)), d_resid(nb * sizeof(double)),
         d_part((size_t)nb * ntile * sizeof(XPart<R>));
     int* list[2] = {d_list.as<int>(), d_list.as<int>() + nb};

@@ -28,6 +28,18 @@ static thread_local Ctx* t_alloc_ctx = nullptr;
 AllocScope::AllocScope(Ctx* c) : prev(t_alloc_ctx) { t_alloc_ctx = c; }
 AllocScope::~AllocScope() { t_alloc_ctx = prev; }
 
+static thread_local cudaStream_t t_tmp_stream = nullptr;
+static thread_local bool t_tmp_on = false;
+
+TmpScope::TmpScope(cudaStream_t s) : prev(t_tmp_stream), prev_on(t_tmp_on) {
+    t_tmp_stream = s;
+    t_tmp_on = true;
+}
+TmpScope::~TmpScope() {
+    t_tmp_stream = prev;
+    t_tmp_on = prev_on;
+}
+
 void DevBuf::alloc(size_t b) {
     release();
     if (b == 0) b = 1;
@@ -41,7 +53,16 @@ void DevBuf::alloc(size_t b) {
                                   std::to_string(cap) + " bytes");
         }
     }
-    cudaError_t e = cudaMalloc(&p, b);
+    // (the null stream names no stream to free on: such a buffer is not pooled)
+    const bool pooled = tmp && t_tmp_on && t_tmp_stream && c && c->pool && b <= TmpBuf::kPoolMax;
+    cudaError_t e = pooled ? cudaMallocFromPoolAsync(&p, b, c->pool, t_tmp_stream) : cudaMalloc(&p, b);
+    if (e == cudaErrorMemoryAllocation && c && c->pool) {  // give back what the pool keeps and try again
+        cudaGetLastError();
+        cudaStreamSynchronize(pooled ? t_tmp_stream : c->stream);
+        cudaMemPoolTrimTo(c->pool, 0);
+        e = pooled ? cudaMallocFromPoolAsync(&p, b, c->pool, t_tmp_stream) : cudaMalloc(&p, b);
+    }
+    if (e == cudaSuccess && pooled) stream = t_tmp_stream;
     if (e != cudaSuccess) {
         p = nullptr;
         if (c) c->allocated.fetch_sub((int64_t)b);
@@ -59,12 +80,14 @@ void DevBuf::alloc(size_t b) {
 
 void DevBuf::release() {
     if (p) {
-        cudaFree(p);
+        if (stream) cudaFreeAsync(p, stream);
+        else cudaFree(p);
         if (owner) owner->allocated.fetch_sub((int64_t)bytes);
     }
     p = nullptr;
     bytes = 0;
     owner = nullptr;
+    stream = nullptr;
 }
 
 // ---------------------------------------------------------------------------

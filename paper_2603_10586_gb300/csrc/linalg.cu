@@ -294,7 +294,7 @@ void invert_self_blocks(Op& op) {
     // shared memory, then pivots, permutation, status and one barrier counter per type
     const size_t nz = 2 * (size_t)np + (in_smem ? 0 : (size_t)G * max_cols * np);
     const size_t ni = 3 * (size_t)np + 1 + op.T;
-    DevBuf buf(nz * sizeof(double2) + ni * sizeof(int));
+    TmpBuf buf(nz * sizeof(double2) + ni * sizeof(int));
     double2* cb = buf.as<double2>();
     double2* work = in_smem ? nullptr : cb + 2 * (size_t)np;
     int* piv = reinterpret_cast<int*>(cb + nz);

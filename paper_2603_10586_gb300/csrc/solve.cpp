@@ -48,11 +48,11 @@ struct Gmres {
     int64_t n;
     int m, nrhs, n_sm;
     bool c64;  // inner applies on float32 vectors
-    DevBuf V, H, g, cs, sn, h, y, part, npart, nsq, rpart, inv, cycling, reorth, jdone, cols, iters, done, beta0, beta, res,
+    TmpBuf V, H, g, cs, sn, h, y, part, npart, nsq, rpart, inv, cycling, reorth, jdone, cols, iters, done, beta0, beta, res,
         rnorm,
         bnorm, hist, ctr, col_lo, col_len, col_voff, colr, colr_cycle, col_prob;
     std::vector<int2> h_colr;
-    DevBuf Xg, Yg, Xl, T, Rl, Wl, W, Rf, enorm, ubound;
+    TmpBuf Xg, Yg, Xl, T, Rl, Wl, W, Rf, enorm, ubound;
     KrylovArgs a{};
     std::map<int, CycleGraph> graphs;
     int* h_pinned = nullptr;  // [KR_NCTR + nrhs] host-visible copy of counters and done flags
@@ -556,10 +556,11 @@ int solve(Op& op, const vie_incident* inc, int nrhs, const vie_solve_opts* o, vo
     cudaStream_t s = op.ctx->stream;
     const int64_t n = op.n();
     double t0 = now_s();
-    DevBuf b((size_t)n * nrhs * sizeof(double2));
+    TmpScope tmp(s);
+    TmpBuf b((size_t)n * nrhs * sizeof(double2));
     const IncidentDev w = upload_incident(op, inc, nrhs, s);
     rhs_kernel_launch(op, w.khat, w.pol, nrhs, b.p, n, s);
-    DevBuf xdev;
+    TmpBuf xdev;
     double2* X;
     if (o->out_on_device) X = static_cast<double2*>(I_out);
     else {
