@@ -9,7 +9,8 @@
 //   phase 2:  P[:, col]  = Q t[:, col]          (m x rank) (rank x columns)
 //   phase 3:  F_a        = sum of the P rows of atom a, in its entry list's order
 // An item is one class, up to kTileMembers of its members and, in phase 1, up
-// to 64 rows and Op::tile_seg columns of R (the segments' partial t are added in
+// to 64 rows (fewer on small operators and in complex128, see build_apply_lists)
+// and Op::tile_seg columns of R (the segments' partial t are added in
 // order where phase 2 reads them, so a long row is neither a long chain nor a
 // late CTA), in phase 2 up to 256 rows of Q.  Every output element is written by
 // one thread and every sum has a fixed order: the result does not depend on the
@@ -27,10 +28,12 @@
 //
 // Measured on one GB300 (fused apply, against the kernels that read a factor once
 // per four copies of one right-hand side or once per four right-hand sides):
-//   16 x 16 array of 6^3 cubes, 1 column, complex float32    953 -> 588 us
+//   4 x 4 array of 3^3 cubes, 1 column, complex float32       38 -> 32 us
+//   16 x 16 array of 6^3 cubes, 1 column, complex float32    953 -> 533 us
 //   28 x 28 array of 3^3 cubes, 5 columns, complex float32  4078 -> 1142 us
 //   16 x 16 array of 4^3 cubes, 24 columns, double-float    18.1 -> 15.3 ms (far part)
-//   12 x 12 array of 3^3 cubes, 3 columns, complex float64  3837 -> 2590 us
+//   12 x 12 array of 3^3 cubes, 3 columns, complex float64  3837 -> 2108 us
+//    8 x 8 array of 3^3 cubes, 1 column, complex float64     642 -> 447 us
 #include <algorithm>
 #include <atomic>
 
@@ -44,7 +47,10 @@ namespace vie {
 namespace {
 
 constexpr int kThr = 128;    // four warps
-constexpr int kTM = 64;      // rows per tile
+template <class TF> constexpr bool kWide = std::is_same<TF, double2>::value;
+// rows per tile of phase 1, and per warp of phase 2
+template <class TF> constexpr int kTM1 = kWide<TF> ? kTileRows1Wide : kTileRows1;
+template <class TF> constexpr int kTM2 = kWide<TF> ? kTileRows2Wide : kTileRows2 / 4;
 
 // Staged operands: A1 [row][K], B [column][K] (K contiguous, as in memory) with
 // one 16-byte unit of padding per row, so that threads a row apart read other
@@ -56,31 +62,38 @@ struct Shape1 {
     static constexpr int KC = WN == 4 ? 16 : 32;     // K values per stage
     static constexpr int KG = KC / WK;               // of those, per K group
     static constexpr int LA = KC + kE<TF>, LB = KC + kE<TX>;
-    static constexpr size_t a_pad = (size_t)kTM * LA * sizeof(TF);
+    static constexpr size_t a_pad = (size_t)kTM1<TF> * LA * sizeof(TF);
     static constexpr size_t stage = a_pad + (size_t)TN * LB * sizeof(TX);
 };
 // phase 2: RW warps down the rows, CW = 4 / RW side by side
 template <class TF, class TX, int RW, int J>
 struct Shape2 {
     static constexpr int CW = 4 / RW, TN = 2 * J * CW, KC = 8;
-    static constexpr int LA = kTM * RW, LB = KC + kE<TX>;
+    static constexpr int LA = kTM2<TF> * RW, LB = KC + kE<TX>;
     static constexpr size_t a_pad = (size_t)KC * LA * sizeof(TF);
     static constexpr size_t stage = a_pad + (size_t)TN * LB * sizeof(TX);
 };
+// complex128 asks for more than it uses, so that an SM holds two CTAs of phase 1
+// and three of phase 2, which keep its float64 units busy, and takes the next
+// when one is done (8 x 8 array of 3^3 cubes, 1 column: 575 us with all it can hold, 447 so)
+constexpr size_t kWideSmem1 = 84 << 10, kWideSmem2 = 68 << 10;
 template <class TF, class TX> constexpr size_t smem_bytes(int phase) {
     constexpr int J = kJ<TX>;
+    if (kWide<TF> && phase == 1) return kWideSmem1;
     if (phase == 1)
         return 2 * std::max({Shape1<TF, TX, 4, J>::stage, Shape1<TF, TX, 2, J>::stage, Shape1<TF, TX, 1, J>::stage});
+    if (kWide<TF>) return kWideSmem2;
     return 2 * std::max({Shape2<TF, TX, 4, J>::stage, Shape2<TF, TX, 2, J>::stage, Shape2<TF, TX, 1, J>::stage});
 }
 
+static_assert(2 * std::max({Shape1<double2, double2, 4, 4>::stage, Shape1<double2, double2, 2, 4>::stage,
+                            Shape1<double2, double2, 1, 4>::stage}) <= kWideSmem1 &&
+              2 * Shape2<double2, double2, 1, 4>::stage <= kWideSmem2);
+
 struct TileArgs {
-    const FarBlockDev* blocks;
     const int* batoms;
     const FarTile* items;
-    const int* cmem;
-    const long long* toff;   // per block: its t in the segment layout
-    const long long* poff;   // per block: its rows of P
+    const FarMember* mem;
     const int2* colr;
     int np, rhs0, nrhs;      // right-hand sides [rhs0, rhs0 + nrhs) of the call in this pass
     int64_t ldx, ldt, ldp;
@@ -93,10 +106,10 @@ struct Cols {
     // column -> (member, right-hand side); exact: columns stay below 2^16
     __device__ __forceinline__ int member(int col) const { return (int)(((float)col + 0.5f) * inv); }
 };
-__device__ __forceinline__ Cols cols_of(const TileArgs& a, const FarTile& it, int prob) {
+__device__ __forceinline__ Cols cols_of(const TileArgs& a, const FarTile& it) {
     int lo = a.rhs0, hi = a.rhs0 + a.nrhs;
     if (a.colr) {
-        const int2 r = a.colr[prob];
+        const int2 r = a.colr[it.prob];
         lo = max(lo, r.x);
         hi = min(hi, r.y);
     }
@@ -108,8 +121,8 @@ __device__ __forceinline__ Cols cols_of(const TileArgs& a, const FarTile& it, in
 // phase 1, columns [q0, q0 + TN) of the item
 // ---------------------------------------------------------------------------
 template <class TF, class TX, int WN, int J, int RA>
-__device__ void tile1(unsigned char* smem, const TileArgs& a, const FarTile& it, const FarBlockDev& B, const Cols& C,
-                      int q0, const TF* __restrict__ fac, const TX* __restrict__ x, TX* __restrict__ t) {
+__device__ void tile1(unsigned char* smem, const TileArgs& a, const FarTile& it, const Cols& C, int q0,
+                      const TF* __restrict__ fac, const TX* __restrict__ x, TX* __restrict__ t) {
     using S = Shape1<TF, TX, WN, J>;
     using TA = typename AccOf<TX>::t;
     constexpr int EA = kE<TF>, EB = kE<TX>;
@@ -118,10 +131,10 @@ __device__ void tile1(unsigned char* smem, const TileArgs& a, const FarTile& it,
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wn = warp % WN, wk = warp / WN, tr = lane & 15, tc = lane >> 4;
     const int ka = tid % UA * EA, pa = tid / UA, kb = tid % UB * EB, pb = tid / UB;
-    const int* mem = a.cmem + it.first;
+    const FarMember* mem = a.mem + it.first;
     const int nst = (it.k1 - it.k0 + S::KC - 1) / S::KC;
-    const TF* RH = fac + B.rh_off + (int64_t)(it.row0 + pa) * B.n + it.k0 + ka;
-    const int64_t rstep = (int64_t)RA_ * B.n;
+    const TF* RH = fac + it.off + (int64_t)(it.row0 + pa) * it.ld + it.k0 + ka;
+    const int64_t rstep = (int64_t)RA_ * it.ld;
     // the columns that this thread stages: pb, pb + RB, ...
     constexpr int NB = (S::TN + RB - 1) / RB;
     const TX* xc[NB];
@@ -133,7 +146,7 @@ __device__ void tile1(unsigned char* smem, const TileArgs& a, const FarTile& it,
         const bool ok = q < S::TN && col < C.n;
         const int j = ok ? C.member(col) : 0, c = ok ? col - j * C.nc : 0;
         xc[u] = x + (int64_t)(C.c0 + c) * a.ldx;
-        Sc[u] = a.batoms + a.blocks[mem[j]].s_off;
+        Sc[u] = a.batoms + mem[j].s_off;
         live |= ok ? 1u << u : 0u;
     }
     // (k1, the atoms' sizes and the segments are even, so a unit never straddles)
@@ -218,7 +231,7 @@ __device__ void tile1(unsigned char* smem, const TileArgs& a, const FarTile& it,
             const int col = q0 + wn * 2 * J + tc + 2 * j;
             if (col < C.n) {
                 const int m = C.member(col), c = col - m * C.nc;
-                TX* out = t + a.toff[mem[m]] + (int64_t)it.seg * B.rank + it.row0 + (int64_t)(C.c0 + c - a.rhs0) * a.ldt;
+                TX* out = t + mem[m].toff + (int64_t)it.seg * it.rank + it.row0 + (int64_t)(C.c0 + c - a.rhs0) * a.ldt;
 #pragma unroll
                 for (int i = 0; i < RA; ++i)
                     if (tr + 16 * i < it.rows) store(out + tr + 16 * i, acc[i][j]);
@@ -233,26 +246,26 @@ __device__ void tile1(unsigned char* smem, const TileArgs& a, const FarTile& it,
 __device__ __forceinline__ int warp_rows(int rows, int RW) { return ((rows + RW - 1) / RW + 1) / 2 * 2; }
 
 template <class TF, class TX, int RW, int J, int RA>
-__device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it, const FarBlockDev& B, const Cols& C,
-                      int q0, const TF* __restrict__ fac, const TX* __restrict__ t, TX* __restrict__ P) {
+__device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it, const Cols& C, int q0,
+                      const TF* __restrict__ fac, const TX* __restrict__ t, TX* __restrict__ P) {
     using S = Shape2<TF, TX, RW, J>;
     using TA = typename AccOf<TX>::t;
     constexpr int KR = kThr / S::KC;  // columns of t staged at a time
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wr = warp % RW, wc = warp / RW, tr = lane & 15, tc = lane >> 4;
     const int kk = tid % S::KC, part = tid / S::KC;
-    const int* mem = a.cmem + it.first;
-    const int K = B.rank, nst = (K + S::KC - 1) / S::KC;
+    const FarMember* mem = a.mem + it.first;
+    const int K = it.rank, nst = (K + S::KC - 1) / S::KC;
     constexpr int EA = kE<TF>;
     const int pw = warp_rows(it.rows, RW);
     // factor: units of EA rows, LA / EA of them per K value, KA K values at a time
     // (a tile of 256 rows x 8 bytes is exactly one K value of the CTA)
     constexpr int UR = S::LA / EA, KA = kThr / UR > 0 ? kThr / UR : 1, NU = (UR + kThr - 1) / kThr;
     const int ur = (tid % UR) * EA, uk = tid / UR;
-    const TF* Q = fac + B.q_off + it.row0 + ur + (int64_t)uk * B.m;
+    const TF* Q = fac + it.off + it.row0 + ur + (int64_t)uk * it.ld;
     auto fill_a = [&](int s) {
         TF* As = reinterpret_cast<TF*>(smem + (s & 1) * S::stage) + uk * S::LA + ur;
-        const TF* src = Q + (int64_t)s * S::KC * B.m;
+        const TF* src = Q + (int64_t)s * S::KC * it.ld;
 #pragma unroll
         for (int k = 0; k < S::KC; k += KA) {
 #pragma unroll
@@ -260,7 +273,7 @@ __device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it,
                 const bool ok = s * S::KC + k + uk < K && ur + h * kThr * EA < it.rows;
                 cp_async16(As + k * S::LA + h * kThr * EA, ok ? src + h * kThr * EA : fac, ok);
             }
-            src += (int64_t)KA * B.m;
+            src += (int64_t)KA * it.ld;
         }
         cp_commit();
     };
@@ -272,7 +285,7 @@ __device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it,
         const int q = part + u * KR, col = q0 + q;
         const bool ok = q < S::TN && col < C.n;
         const int j = ok ? C.member(col) : 0, c = ok ? col - j * C.nc : 0;
-        tb[u] = t + a.toff[mem[j]] + (int64_t)(C.c0 + c - a.rhs0) * a.ldt + kk;
+        tb[u] = t + mem[j].toff + (int64_t)(C.c0 + c - a.rhs0) * a.ldt + kk;
         live |= ok ? 1u << u : 0u;
     }
     TX bv[NB];
@@ -289,6 +302,8 @@ __device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it,
     };
     TA acc[RA][J];
     zero_acc(acc);
+    const int rows = min(pw, it.rows - wr * pw);          // (none for a warp past the last row)
+    const bool busy = rows > 0 && q0 + wc * 2 * J < C.n;  // (nor past the last column)
     fill_a(0);
     load_b(0);
     for (int s = 0; s < nst; ++s) {
@@ -302,18 +317,17 @@ __device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it,
         }
         __syncthreads();
         const unsigned char* st = smem + (s & 1) * S::stage;
-        mma_stage<TF, TX, TA, 2, S::KC, S::LA, S::LB, RA, J>(
+        if (busy) mma_stage<TF, TX, TA, 2, S::KC, S::LA, S::LB, RA, J>(
             reinterpret_cast<const TF*>(st) + wr * pw + EA * tr,
             reinterpret_cast<const TX*>(st + S::a_pad) + (wc * 2 * J + tc) * S::LB, acc);
         __syncthreads();
     }
-    const int rows = min(pw, it.rows - wr * pw);  // (none for a warp past the last row)
 #pragma unroll
     for (int j = 0; j < J; ++j) {
         const int col = q0 + wc * 2 * J + tc + 2 * j;
         if (col < C.n) {
             const int m = C.member(col), c = col - m * C.nc;
-            TX* out = P + a.poff[mem[m]] + it.row0 + wr * pw + (int64_t)(C.c0 + c - a.rhs0) * a.ldp;
+            TX* out = P + mem[m].poff + it.row0 + wr * pw + (int64_t)(C.c0 + c - a.rhs0) * a.ldp;
 #pragma unroll
             for (int i = 0; i < RA; ++i) {
                 const int r = EA == 2 ? 32 * (i >> 1) + 2 * tr + (i & 1) : 16 * i + tr;
@@ -325,16 +339,22 @@ __device__ void tile2(unsigned char* smem, const TileArgs& a, const FarTile& it,
 
 template <class TF, class TX, int PHASE, int W, int J>
 __device__ __forceinline__ void tile_rows(unsigned char* smem, const TileArgs& a, const FarTile& it,
-                                          const FarBlockDev& B, const Cols& C, int q0, const TF* fac, const TX* in,
+                                          const Cols& C, int q0, const TF* fac, const TX* in,
                                           TX* out) {
     const int r = PHASE == 1 ? it.rows : warp_rows(it.rows, W);  // rows of a warp tile
-    if constexpr (PHASE == 1) {
-        if (r > 48) tile1<TF, TX, W, J, 4>(smem, a, it, B, C, q0, fac, in, out);
-        else if (r > 32) tile1<TF, TX, W, J, 3>(smem, a, it, B, C, q0, fac, in, out);
-        else tile1<TF, TX, W, J, 2>(smem, a, it, B, C, q0, fac, in, out);
+    if constexpr (PHASE == 1 && kWide<TF>) {
+        tile1<TF, TX, W, J, 1>(smem, a, it, C, q0, fac, in, out);
+    } else if constexpr (PHASE == 1) {
+        if (r > 48) tile1<TF, TX, W, J, 4>(smem, a, it, C, q0, fac, in, out);
+        else if (r > 32) tile1<TF, TX, W, J, 3>(smem, a, it, C, q0, fac, in, out);
+        else if (r > 16 || kE<TX> > 1) tile1<TF, TX, W, J, 2>(smem, a, it, C, q0, fac, in, out);
+        else if constexpr (kE<TX> == 1) tile1<TF, TX, W, J, 1>(smem, a, it, C, q0, fac, in, out);
+    } else if constexpr (kWide<TF>) {
+        if (r > 16) tile2<TF, TX, W, J, 2>(smem, a, it, C, q0, fac, in, out);
+        else tile2<TF, TX, W, J, 1>(smem, a, it, C, q0, fac, in, out);
     } else {
-        if (r > 32) tile2<TF, TX, W, J, 4>(smem, a, it, B, C, q0, fac, in, out);
-        else tile2<TF, TX, W, J, 2>(smem, a, it, B, C, q0, fac, in, out);
+        if (r > 32) tile2<TF, TX, W, J, 4>(smem, a, it, C, q0, fac, in, out);
+        else tile2<TF, TX, W, J, 2>(smem, a, it, C, q0, fac, in, out);
     }
 }
 
@@ -344,31 +364,33 @@ __global__ void __launch_bounds__(kThr, std::is_same<TX, float4>::value ? 4 : 3)
                                                                         const TX* __restrict__ in,
                                                                         TX* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char tile_smem[];
-    constexpr int J = kJ<TX>, H = J > 4 ? 4 : J;  // columns per thread: full, and for the last few
+    constexpr int J = kJ<TX>, H = J / 2;  // columns per thread: full, and for the last few
     const FarTile it = a.items[blockIdx.x];
-    const FarBlockDev B = a.blocks[a.cmem[it.first]];
-    const Cols C = cols_of(a, it, B.prob);
+    const Cols C = cols_of(a, it);
     if constexpr (PHASE == 1) {
         for (int q = blockIdx.y * 8 * J; q < C.n; q += gridDim.y * 8 * J) {
             const int n = C.n - q;
-            if (n > 4 * J) tile_rows<TF, TX, 1, 4, J>(tile_smem, a, it, B, C, q, fac, in, out);
-            else if (n > 2 * J) tile_rows<TF, TX, 1, 2, J>(tile_smem, a, it, B, C, q, fac, in, out);
-            else if (n > 2 * H) tile_rows<TF, TX, 1, 1, J>(tile_smem, a, it, B, C, q, fac, in, out);
-            else tile_rows<TF, TX, 1, 1, H>(tile_smem, a, it, B, C, q, fac, in, out);
+            if (n > 4 * J) tile_rows<TF, TX, 1, 4, J>(tile_smem, a, it, C, q, fac, in, out);
+            else if (n > 2 * J) tile_rows<TF, TX, 1, 2, J>(tile_smem, a, it, C, q, fac, in, out);
+            else if (n > 2 * H) tile_rows<TF, TX, 1, 1, J>(tile_smem, a, it, C, q, fac, in, out);
+            else tile_rows<TF, TX, 1, 1, H>(tile_smem, a, it, C, q, fac, in, out);
         }
     } else {
-        const int cw = it.rows > 2 * kTM ? 1 : it.rows > kTM ? 2 : 4, tn = 2 * J * cw;
+        const int cw = kWide<TF> ? 4 : it.rows > 2 * kTM2<TF> ? 1 : it.rows > kTM2<TF> ? 2 : 4, tn = 2 * J * cw;
         for (int q = blockIdx.y * tn; q < C.n; q += gridDim.y * tn) {
             const bool half = C.n - q <= 2 * H * cw;
-            if (cw == 1) {
-                if (half) tile_rows<TF, TX, 2, 4, H>(tile_smem, a, it, B, C, q, fac, in, out);
-                else tile_rows<TF, TX, 2, 4, J>(tile_smem, a, it, B, C, q, fac, in, out);
+            if constexpr (kWide<TF>) {
+                if (half) tile_rows<TF, TX, 2, 1, H>(tile_smem, a, it, C, q, fac, in, out);
+                else tile_rows<TF, TX, 2, 1, J>(tile_smem, a, it, C, q, fac, in, out);
+            } else if (cw == 1) {
+                if (half) tile_rows<TF, TX, 2, 4, H>(tile_smem, a, it, C, q, fac, in, out);
+                else tile_rows<TF, TX, 2, 4, J>(tile_smem, a, it, C, q, fac, in, out);
             } else if (cw == 2) {
-                if (half) tile_rows<TF, TX, 2, 2, H>(tile_smem, a, it, B, C, q, fac, in, out);
-                else tile_rows<TF, TX, 2, 2, J>(tile_smem, a, it, B, C, q, fac, in, out);
+                if (half) tile_rows<TF, TX, 2, 2, H>(tile_smem, a, it, C, q, fac, in, out);
+                else tile_rows<TF, TX, 2, 2, J>(tile_smem, a, it, C, q, fac, in, out);
             } else {
-                if (half) tile_rows<TF, TX, 2, 1, H>(tile_smem, a, it, B, C, q, fac, in, out);
-                else tile_rows<TF, TX, 2, 1, J>(tile_smem, a, it, B, C, q, fac, in, out);
+                if (half) tile_rows<TF, TX, 2, 1, H>(tile_smem, a, it, C, q, fac, in, out);
+                else tile_rows<TF, TX, 2, 1, J>(tile_smem, a, it, C, q, fac, in, out);
             }
         }
     }
@@ -401,10 +423,10 @@ __global__ void __launch_bounds__(64) k_tile_seg(const FarBlockDev* __restrict__
 // F[a rows] = sum of the partial products of atom a's (block, slot) entries in
 // list order, eight of them in flight; blockIdx.y = right-hand side of the pass
 template <class TX, class TO>
-__global__ void __launch_bounds__(128) k_tile_sum(const int4* __restrict__ items, int n_items, const int* __restrict__ csr,
-                                                  const int2* __restrict__ ent, const long long* __restrict__ poff,
-                                                  const TX* __restrict__ P, int64_t ldp, int np, TO* __restrict__ F,
-                                                  int64_t ldf, int rhs0, const int2* __restrict__ colr) {
+__global__ void __launch_bounds__(128) k_tile_sum(const int4* __restrict__ items, const int* __restrict__ csr,
+                                                  const long long* __restrict__ pbase, const TX* __restrict__ P,
+                                                  int64_t ldp, int np, TO* __restrict__ F, int64_t ldf, int rhs0,
+                                                  const int2* __restrict__ colr) {
     using TA = typename AccOf<TX>::t;
     const int c = rhs0 + blockIdx.y;
     const int4 item = items[blockIdx.x];
@@ -413,43 +435,44 @@ __global__ void __launch_bounds__(128) k_tile_sum(const int4* __restrict__ items
         const int2 cr = colr[item.w];
         if (c < cr.x || c >= cr.y) return;
     }
-    __shared__ long long base[128];
+    if (row >= item.z) return;
     const TX* Pc = P + (int64_t)blockIdx.y * ldp + row;
-    const bool mine = row < item.z;
     TA acc = acc_zero<TA>();
-    for (int e0 = csr[a]; e0 < csr[a + 1]; e0 += 128) {
-        const int ne = min(128, csr[a + 1] - e0);
-        __syncthreads();
-        if ((int)threadIdx.x < ne) {
-            const int2 en = ent[e0 + threadIdx.x];
-            base[threadIdx.x] = poff[en.x] + (int64_t)en.y * np;
-        }
-        __syncthreads();
-        if (!mine) continue;
-        int e = 0;
-        for (; e + 8 <= ne; e += 8) {
-            TX v[8];
+    int e = csr[a];
+    const int e1 = csr[a + 1];
+    for (; e + 8 <= e1; e += 8) {
+        TX v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = Pc[base[e + u]];
+        for (int u = 0; u < 8; ++u) v[u] = Pc[__ldg(pbase + e + u)];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc_add(acc, as_acc(v[u]));
-        }
-        for (; e < ne; ++e) acc_add(acc, as_acc(Pc[base[e]]));
+        for (int u = 0; u < 8; ++u) acc_add(acc, as_acc(v[u]));
     }
-    if (mine) store(F + (int64_t)a * np + row + (int64_t)c * ldf, acc);
+    for (; e < e1; ++e) acc_add(acc, as_acc(Pc[__ldg(pbase + e)]));
+    store(F + (int64_t)a * np + row + (int64_t)c * ldf, acc);
 }
 
-// right-hand sides per pass: their partial products stay within kTilePass bytes (or one column's)
+// right-hand sides per pass: their partial products stay within kTilePass bytes, or
+// sixteen columns' (few columns leave tiles empty: 11 columns of the 27 x 27 graded
+// array of 4^3 cubes in double-float, one at a time, took 59 ms).  At most 1024,
+// which Cols::member needs.
 int pass_cols(const Op& op, int nrhs, size_t elem) {
     const size_t per = (size_t)std::max<int64_t>(op.part_total, 1) * elem;
-    return (int)std::max<size_t>(1, std::min<size_t>(nrhs, Op::kTilePass / per));
+    return (int)std::min<size_t>(std::min(nrhs, 1024), std::max<size_t>(16, Op::kTilePass / per));
 }
 
 }  // namespace
 
 // The tile kernels read a factor once per group of columns; the per-block kernels
-// once per right-hand side or four of them, but without partial products.
-bool tile_pays(const Op& op, int nrhs) { return op.share_mean * nrhs >= 3.0; }
+// once per right-hand side or four of them, but without partial products.  Without
+// shared factors (gold atoms on a spiral, 3^3 cubes, us): 2 columns pay, 400 atoms 1192 -> 922;
+// one column does not, 500 atoms 795 -> 1206, unless the per-block kernel, a CTA for 128 rows
+// of an atom, has too few CTAs to hide its loads: 60 atoms 218 -> 108, 150 339 -> 281,
+// 200 395 -> 392, 300 523 -> 651.  (complex128 padding costs more: 3 columns.)
+bool tile_pays(const Op& op, int nrhs) {
+    const double least = op.fprec == VIE_C128 || nrhs == 1 ? 3.0 : 2.0;
+    const bool few = op.fprec != VIE_C128 && 2 * op.n_p2_items < 3 * op.ctx->n_sm;
+    return op.share_mean * nrhs >= least || few;
+}
 
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
     const size_t rp = pass_cols(op, nrhs, elem);
@@ -486,8 +509,7 @@ void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nr
     }
     for (int c0 = first; c0 < last; c0 += rp) {
         const int nc = std::min(rp, last - c0);
-        TileArgs a{op.d_blocks.as<FarBlockDev>(), op.d_block_atoms.as<int>(), op.d_c1_items.as<FarTile>(),
-                   op.d_cmem.as<int>(), op.d_ctoff.as<long long>(), op.d_poff.as<long long>(), op.colr, op.np, c0, nc,
+        TileArgs a{op.d_block_atoms.as<int>(), op.d_c1_items.as<FarTile>(), op.d_cmem.as<FarMember>(), op.colr, op.np, c0, nc,
                    ldx, op.ct_total, op.part_total};
         const unsigned gy = (unsigned)std::min((op.tile_group * nc + 8 * kJ<TX> - 1) / (8 * kJ<TX>), 65535);
         if (op.n_c1_items > 0) {
@@ -495,8 +517,8 @@ void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nr
             VIE_CHECK_LAUNCH();
         }
         if (op.n_cseg > 0) {
-            k_tile_seg<TX><<<dim3(op.n_cseg, nc), 64, 0, s>>>(a.blocks, op.d_cseg.as<int>(), a.toff, op.tile_seg, t,
-                                                             op.ct_total);
+            k_tile_seg<TX><<<dim3(op.n_cseg, nc), 64, 0, s>>>(op.d_blocks.as<FarBlockDev>(), op.d_cseg.as<int>(),
+                                                             op.d_ctoff.as<long long>(), op.tile_seg, t, op.ct_total);
             VIE_CHECK_LAUNCH();
         }
         if (op.n_c2_items > 0) {
@@ -505,8 +527,7 @@ void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nr
             VIE_CHECK_LAUNCH();
         }
         k_tile_sum<TX, TO><<<dim3(op.n_p2_items, nc), 128, 0, s>>>(
-            op.d_p2_items.as<int4>(), op.n_p2_items, op.d_p2_csr.as<int>(), op.d_p2_ent.as<int2>(),
-            op.d_poff.as<long long>(), P, op.part_total, op.np, F, ldf, c0, op.colr);
+            op.d_p2_items.as<int4>(), op.d_p2_csr.as<int>(), op.d_pbase.as<long long>(), P, op.part_total, op.np, F, ldf, c0, op.colr);
         VIE_CHECK_LAUNCH();
     }
 }

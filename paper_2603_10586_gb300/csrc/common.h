@@ -211,11 +211,11 @@ struct Op {
     int n_t1_items = 0, n_t2_items = 0, n_cta_tc = 0;
     // register-tile path (apply_tile.cu): blocks with the same factor storage
     // (translated copies) form a class, listed in d_cmem in groups of up to
-    // kTileMembers; phase 1 writes t at d_ctoff[block] (one part per tile_seg
-    // columns of R), phase 2 one partial product per (block, target slot) at
-    // d_poff[block] + slot np
-    DevBuf d_cmem, d_c1_items, d_c2_items, d_cseg, d_ctoff, d_poff, d_ct, d_part;
-    static constexpr size_t kTilePass = (size_t)256 << 20;  // partial products of one pass (or one column's)
+    // kTileMembers; phase 1 writes t (one part per tile_seg columns of R), phase 2
+    // one partial product per (block, target slot), at d_pbase for the entries of
+    // the atoms' lists
+    DevBuf d_cmem, d_c1_items, d_c2_items, d_cseg, d_ctoff, d_pbase, d_ct, d_part;
+    static constexpr size_t kTilePass = (size_t)2 << 30;  // partial products of one pass (or sixteen columns')
     int n_c1_items = 0, n_c2_items = 0, tile_seg = 512;
     int n_cseg = 0, tile_group = 1;  // blocks with several segments, members of the largest group
     int64_t ct_total = 0, part_total = 0;  // entries of t and of the partial products per right-hand side
@@ -311,12 +311,20 @@ struct AllocScope {
     ~AllocScope();
 };
 
-// one item of the register-tile apply: the members cmem[first .. first + nm) of
-// a class, rows [row0, row0 + rows) of R (phase 1, columns [k0, k1), segment seg)
-// or of Q (phase 2)
+// one item of the register-tile apply: the members [first, first + nm) of a
+// class, rows [row0, row0 + rows) of R (phase 1, columns [k0, k1), segment seg; factor
+// at off, ld = n) or of Q (phase 2; ld = m).  The records carry what the kernels
+// need of the blocks, so that a CTA starts after two dependent loads.
 struct FarTile {
-    int first, nm, row0, rows, k0, k1, seg, pad;
+    int first, nm, row0, rows, k0, k1, seg, prob, rank, ld;
+    long long off;
 };
+struct FarMember {
+    long long toff, poff;  // its t (segment layout), its rows of the partial products
+    int s_off, pad;        // its source atoms
+};
+// rows of an item in phases 1 and 2, at most: complex64 factors, complex128 factors
+constexpr int kTileRows1 = 64, kTileRows2 = 256, kTileRows1Wide = 16, kTileRows2Wide = 32;
 constexpr int kTileMembers = 64;  // members per item: a full group fills 64-column tiles whatever the right-hand-side count
 
 // ---- warp-specialised tensor-core apply (apply_ws.cu) -----------------------

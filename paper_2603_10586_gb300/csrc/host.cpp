@@ -446,8 +446,8 @@ void build_apply_lists(Op& op) {
     op.d_ws_q.release();
 
     // register-tile path: classes of blocks with the same factor storage, in
-    // groups of up to kTileMembers members; phase 1 items of up to 64 rows and
-    // tile_seg columns of R, phase 2 items of up to 256 rows of Q.  Rows are cut
+    // groups of up to kTileMembers members; phase 1 items of up to rows1 rows and
+    // tile_seg columns of R, phase 2 items of up to rows2 rows of Q.  Rows are cut
     // into equal pieces (96 = 48 + 48), in storage order: the coarse levels'
     // long items come first.
     {
@@ -466,6 +466,26 @@ void build_apply_lists(Op& op) {
         op.tile_seg = 128;
         while (op.tile_seg < 512 && 2.0 * op.tile_seg * 64 * 16 * 16 * op.ctx->n_sm <= work) op.tile_seg *= 2;
         const int seg_len = op.tile_seg;
+        // Rows per item.  complex64: 64 of R and 256 of Q, or 32 and 64 where shared
+        // factors leave an SM fewer than eight items of phase 1 (one column, us: 4 x 4
+        // array of 3^3 cubes 36.0 -> 31.9, 8 x 8 70 -> 55, 16 x 16 153 -> 131; above, the
+        // factor's staging counts: 20 x 20 222 -> 226, 28 x 28 of 4^3 763 -> 939; so it does
+        // where no two blocks share: 35 atoms of the spiral, 3 columns, 64 -> 75).
+        // complex128: 16 and 32 always; a product takes its SM's two float64 units
+        // for so long that copies cost nothing and the last items' length everything
+        // (8 x 8 array of 3^3 cubes, 1 column: 817 -> 447 us, 12 x 12, 3 columns: 2476 -> 2108).
+        const bool wide = op.fprec == VIE_C128;
+        int64_t nmem = 0, n64 = 0;
+        for (const auto& kv : cls) {
+            const auto& b = op.blocks[kv.second[0]];
+            const int64_t cnt = (int64_t)kv.second.size();
+            nmem += cnt;
+            n64 += (cnt + kTileMembers - 1) / kTileMembers * ((b.n + seg_len - 1) / seg_len) * ((b.rank + kTileRows1 - 1) / kTileRows1);
+        }
+        op.share_mean = cls.empty() ? 1.0 : (double)nmem / (double)cls.size();
+        const bool fine = op.share_mean >= 3.0 && n64 < 8 * (int64_t)op.ctx->n_sm;
+        const int rows1 = wide ? kTileRows1Wide : fine ? 32 : kTileRows1;
+        const int rows2 = wide ? kTileRows2Wide : fine ? 64 : kTileRows2;
         std::vector<long long> poff(std::max(nb, 1), 0), ctoff(std::max(nb, 1), 0);
         std::vector<int> cseg;
         int64_t ptot = 0, ctot = 0;
@@ -478,13 +498,11 @@ void build_apply_lists(Op& op) {
             ctot += (int64_t)b.rank * ((b.n + seg_len - 1) / seg_len);
             if (b.n > seg_len) cseg.push_back(i);
         }
-        std::vector<int> cmem;
+        std::vector<FarMember> cmem;
         std::vector<FarTile> c1, c2;
-        int64_t nmem = 0;
         op.tile_group = 1;
         for (const auto& kv : cls) {
             const auto& mem = kv.second;
-            nmem += (int64_t)mem.size();
             const auto& b = op.blocks[mem[0]];
             auto tiles = [](int rows, int most, auto&& f) {  // equal pieces of at most `most` rows
                 const int nt = (rows + most - 1) / most, per = ((rows + nt - 1) / nt + 1) / 2 * 2;  // even: 16-byte copies
@@ -494,16 +512,21 @@ void build_apply_lists(Op& op) {
                 const int first = (int)cmem.size();
                 const int cnt = (int)std::min<size_t>(kTileMembers, mem.size() - g);
                 op.tile_group = std::max(op.tile_group, cnt);
-                for (int j = 0; j < cnt; ++j) cmem.push_back(mem[g + j]);
+                for (int j = 0; j < cnt; ++j) {
+                    const int i = mem[g + j];
+                    cmem.push_back(FarMember{ctoff[i], poff[i], op.blocks[i].s_off, 0});
+                }
+                const int prob = kv.first.second;
                 for (int seg = 0; seg * seg_len < b.n; ++seg)
-                    tiles(b.rank, 64, [&](int r0, int rows) {
+                    tiles(b.rank, rows1, [&](int r0, int rows) {
                         c1.push_back(FarTile{first, cnt, r0, rows, seg * seg_len, std::min(b.n, (seg + 1) * seg_len),
-                                             seg, 0});
+                                             seg, prob, b.rank, b.n, (long long)b.rh_off});
                     });
-                tiles(b.m, 256, [&](int r0, int rows) { c2.push_back(FarTile{first, cnt, r0, rows, 0, 0, 0, 0}); });
+                tiles(b.m, rows2, [&](int r0, int rows) {
+                    c2.push_back(FarTile{first, cnt, r0, rows, 0, 0, 0, prob, b.rank, b.m, (long long)b.q_off});
+                });
             }
         }
-        op.share_mean = cls.empty() ? 1.0 : (double)nmem / (double)cls.size();
         op.part_total = ptot;
         op.ct_total = ctot;
         op.n_c1_items = (int)c1.size();
@@ -512,8 +535,10 @@ void build_apply_lists(Op& op) {
         upload(op.d_c2_items, c2.empty() ? std::vector<FarTile>{FarTile{}} : c2);
         op.n_cseg = (int)cseg.size();
         upload(op.d_cseg, cseg);
-        upload(op.d_cmem, cmem.empty() ? std::vector<int>{0} : cmem);
-        upload(op.d_poff, poff);
+        upload(op.d_cmem, cmem.empty() ? std::vector<FarMember>{FarMember{}} : cmem);
+        std::vector<long long> pbase;  // per entry of the atoms' (block, slot) lists
+        for (const int2& e : flat) pbase.push_back(poff[e.x] + (long long)e.y * op.np);
+        upload(op.d_pbase, pbase);
         upload(op.d_ctoff, ctoff);
         op.d_part.release();  // sized on first use (tile_reserve)
         op.d_ct.release();

@@ -173,7 +173,9 @@ constexpr int kGemmThr = 128;
 template <class T, int WN, int RA, int J>
 struct GemmShape {
     static constexpr int WK = 4 / WN, TM = 16 * RA, TN = 2 * J * WN;
-    static constexpr int KC = 16, KG = KC / WK;
+    // (the narrow tile of small arrays takes its K range in few, longer stages: their
+    // latency is all there is)
+    static constexpr int KC = RA == 2 ? 512 / (int)sizeof(T) : 16, KG = KC / WK;
     static constexpr int LA = TM, LB = KC + kE<T>;  // A [K][row], B [column][K]
     static constexpr size_t a_pad = (size_t)KC * LA * sizeof(T);
     static constexpr size_t stage = a_pad + (size_t)TN * LB * sizeof(T);

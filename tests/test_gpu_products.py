@@ -109,3 +109,13 @@ def test_precond(ns, nv, nrhs, precision):
     assert err < (1e-5 if precision == "C64" else 1e-13)
     op.close()
     ctx.close()
+
+
+# short items (16 rows of R, 32 of Q in complex128; 32 and 64 where shared factors
+# leave few items) and long ones (64 and 256) with one to two column tiles
+@pytest.mark.parametrize("array,tol,precision,nrhs", [
+    ("square 5 3", 1e-4, "C128", 1), ("spiral 12 2", 1e-3, "C128", 4), ("square 3 4", 1e-6, "C128", 9),
+    ("square 7 3", 1e-5, "C64", 1), ("square 5 4", 1e-3, "C64", 6), ("spiral 25 3", 1e-5, "C64", 9),
+    ("square 18 3", 1e-4, "C64", 1), ("square 6 3", 1e-2, "C64_ACC64", 2)])
+def test_apply_item_rows(array, tol, precision, nrhs):
+    test_apply(array, tol, precision, nrhs)
