@@ -30,9 +30,9 @@
 // per four copies of one right-hand side or once per four right-hand sides):
 //   4 x 4 array of 3^3 cubes, 1 column, complex float32       38 -> 32 us
 //   16 x 16 array of 6^3 cubes, 1 column, complex float32    953 -> 533 us
-//   28 x 28 array of 3^3 cubes, 5 columns, complex float32  4078 -> 1142 us
-//   16 x 16 array of 4^3 cubes, 24 columns, double-float    18.1 -> 15.3 ms (far part)
-//   12 x 12 array of 3^3 cubes, 3 columns, complex float64  3837 -> 2108 us
+//   28 x 28 array of 3^3 cubes, 5 columns, complex float32  4105 -> 1132 us
+//   16 x 16 array of 4^3 cubes, 24 columns, double-float    20.9 -> 17.3 ms
+//   12 x 12 array of 3^3 cubes, 3 columns, complex float64  3840 -> 2102 us
 //    8 x 8 array of 3^3 cubes, 1 column, complex float64     642 -> 447 us
 #include <algorithm>
 #include <atomic>
