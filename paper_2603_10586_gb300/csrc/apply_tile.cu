@@ -509,8 +509,9 @@ void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nr
     }
     for (int c0 = first; c0 < last; c0 += rp) {
         const int nc = std::min(rp, last - c0);
-        TileArgs a{op.d_block_atoms.as<int>(), op.d_c1_items.as<FarTile>(), op.d_cmem.as<FarMember>(), op.colr, op.np, c0, nc,
-                   ldx, op.ct_total, op.part_total};
+        const bool longest = op.tile_long && (kWide<TF> || (kE<TX> > 1 && nc <= 2));  // (build_apply_lists)
+        TileArgs a{op.d_block_atoms.as<int>(), (longest ? op.d_c1_long : op.d_c1_items).as<FarTile>(),
+                   op.d_cmem.as<FarMember>(), op.colr, op.np, c0, nc, ldx, op.ct_total, op.part_total};
         const unsigned gy = (unsigned)std::min((op.tile_group * nc + 8 * kJ<TX> - 1) / (8 * kJ<TX>), 65535);
         if (op.n_c1_items > 0) {
             k_tile<TF, TX, 1><<<dim3(op.n_c1_items, gy), kThr, smem1, s>>>(a, op.fac<TF>(), x, t);
@@ -522,7 +523,7 @@ void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nr
             VIE_CHECK_LAUNCH();
         }
         if (op.n_c2_items > 0) {
-            a.items = op.d_c2_items.as<FarTile>();
+            a.items = (longest ? op.d_c2_long : op.d_c2_items).as<FarTile>();
             k_tile<TF, TX, 2><<<dim3(op.n_c2_items, gy), kThr, smem2, s>>>(a, op.fac<TF>(), t, P);
             VIE_CHECK_LAUNCH();
         }

@@ -215,6 +215,8 @@ struct Op {
     // one partial product per (block, target slot), at d_pbase for the entries of
     // the atoms' lists
     DevBuf d_cmem, d_c1_items, d_c2_items, d_cseg, d_ctoff, d_pbase, d_ct, d_part;
+    DevBuf d_c1_long, d_c2_long;  // the items, longest first (tile_long)
+    bool tile_long = false;
     static constexpr size_t kTilePass = (size_t)2 << 30;  // partial products of one pass (or sixteen columns')
     int n_c1_items = 0, n_c2_items = 0, tile_seg = 512;
     int n_cseg = 0, tile_group = 1;  // blocks with several segments, members of the largest group

@@ -533,6 +533,24 @@ void build_apply_lists(Op& op) {
         op.n_c2_items = (int)c2.size();
         upload(op.d_c1_items, c1.empty() ? std::vector<FarTile>{FarTile{}} : c1);
         upload(op.d_c2_items, c2.empty() ? std::vector<FarTile>{FarTile{}} : c2);
+        // The same, longest first, for one or two columns of complex float32 on shared
+        // factors and for complex128.  The storage order ends with the fine levels, whose
+        // groups are the largest: with more items than resident CTAs these started last and set
+        // the time (arrays of 3^3 cubes, 1 column, us: 7 x 7 70 -> 52, 11 x 11 119 -> 90, 28 x 28
+        // 396 -> 369; complex128, 7 x 7, 471 -> 358).  With more columns, and in double-float,
+        // an item is whole tiles whatever its class, and the storage order, in which
+        // neighbours share x and factors, is up to 2% faster (16 x 16, 12 columns, 628 against
+        // 635 us; double-float, 16 x 16 of 4^3, 1 column, 922 against 942); so it is without
+        // shared factors (300 atoms of the spiral, 2 columns, 655 against 660).
+        op.tile_long = wide || op.share_mean >= 3.0;
+        if (!op.tile_long) c1.clear(), c2.clear();
+        auto by_cost = [](std::vector<FarTile>& v, auto&& cost) {
+            std::stable_sort(v.begin(), v.end(), [&](const FarTile& a, const FarTile& b) { return cost(a) > cost(b); });
+        };
+        by_cost(c1, [](const FarTile& t) { return (long long)(t.k1 - t.k0) * (8 + t.nm); });
+        by_cost(c2, [](const FarTile& t) { return (long long)t.rank * (8 + t.nm); });
+        upload(op.d_c1_long, c1.empty() ? std::vector<FarTile>{FarTile{}} : c1);
+        upload(op.d_c2_long, c2.empty() ? std::vector<FarTile>{FarTile{}} : c2);
         op.n_cseg = (int)cseg.size();
         upload(op.d_cseg, cseg);
         upload(op.d_cmem, cmem.empty() ? std::vector<FarMember>{FarMember{}} : cmem);

@@ -1,0 +1,36 @@
+"""Order of the register tiles' items: with more items than resident CTAs the long
+ones have to start first.  The 7 x 7 array has fewer products than the 8 x 8 array
+but 1.7 times the items; with its long items last it took 1.28 times as long."""
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+def _apply_us(ns):
+    import numpy as np
+    import torch
+    from paper_2603_10586_gb300 import vie
+    ctx = vie.Context(0)
+    op = vie.Operator(ctx, workloads.square_array(ns, 3))
+    op.compress(1e-4, vie.C64)
+    x = torch.from_numpy(workloads.random_complex(op.n, 3).reshape(-1).astype(np.complex64)).cuda()
+    y = torch.empty_like(x)
+    s = torch.cuda.Stream()
+    times = []
+    for _ in range(8):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record(s)
+        for _ in range(200):
+            op.apply(x.data_ptr(), y.data_ptr(), 1, vie.C64, 0, stream=s.cuda_stream)
+        b.record(s)
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) * 5.0)
+    op.close()
+    ctx.close()
+    return min(times[1:])
+
+
+def test_smaller_array_is_not_slower():
+    assert _apply_us(7) < 1.12 * _apply_us(8)
