@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(256) k_sphere_sum(const double2* __restrict__ 
 // the sums S = sum w g, S_d = sum w x_d g and K = sum w grad g are formed, and a
 // column takes them with its six face currents.  The sums over z run
 // innermost, so a Gauss point adds to four sums instead of seven.
-// part[((z npts + p) C + c) 3 + d], chunk z of the atoms.
+// part[((z npts + p) C + c) 3 + d], chunk z of the atoms, points of this pass.
 // ---------------------------------------------------------------------------
 struct GreenSum {
     double2 g, f;  // exp(-j k R) / R and (1 + j k R) g / R^2 (both times 4 pi, the sign of grad g apart)
@@ -372,13 +372,22 @@ __global__ void __launch_bounds__(256) k_near(DevMesh m, Geo geo, double k, cons
     }
 }
 
-__global__ void k_near_finish(const double2* __restrict__ part, int npts, int C, int nz, double2* __restrict__ out) {
+// points [p0, p0 + npts) of `total`
+__global__ void k_near_finish(const double2* __restrict__ part, int npts, int C, int nz, int64_t p0, int64_t total,
+                              double2* __restrict__ out) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= npts * C * 3) return;
     const int d = t % 3, c = (t / 3) % C, p = t / (3 * C);
     double2 s = make_double2(0, 0);
     for (int z = 0; z < nz; ++z) s += part[(((size_t)z * npts + p) * C + c) * 3 + d];
-    out[((size_t)c * npts + p) * 3 + d] = s;
+    out[(c * total + p0 + p) * 3 + d] = s;
+}
+
+// points or directions of one pass: a chunk of atoms' partial sums stay within 32 MB,
+// and their number within 32 bits (as many sums as outputs in one pass would double
+// what a call with many points holds)
+int sum_cols(int nrhs, int npts) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(npts, ((int64_t)32 << 20) / (48ll * nrhs)));
 }
 
 void grow(DevBuf& b, size_t bytes) {
@@ -438,7 +447,7 @@ void rhs_kernel_launch(Op& op, const double* d_khat, const double* d_pol, int nr
 // far-field amplitudes of nrhs currents in npts directions: d_out[(c npts + p) 3 + d]
 void far_field_launch(Op& op, const void* d_I, int nrhs, const double* d_dirs, int npts, void* d_out,
                       cudaStream_t s) {
-    const int wc = table_cols(op, npts), groups = (nrhs + kRC - 1) / kRC;
+    const int wc = std::min(table_cols(op, npts), sum_cols(nrhs, npts)), groups = (nrhs + kRC - 1) / kRC;
     for (int w0 = 0; w0 < npts; w0 += wc) {
         const int W = std::min(wc, npts - w0);
         double2* ph;
@@ -485,18 +494,20 @@ void sphere_sum_launch(const void* d_F, const double* d_wt, int npts, int nrhs, 
 }
 
 void near_field_launch(Op& op, const void* d_I, int nrhs, const double* d_pts, int npts, void* d_out, cudaStream_t s) {
-    const int groups = (nrhs + kRC - 1) / kRC;
-    int nz = atom_chunks(op, (int64_t)npts * groups, 1);
+    const int pc = sum_cols(nrhs, npts), groups = (nrhs + kRC - 1) / kRC;
+    int nz = atom_chunks(op, (int64_t)pc * groups, 1);
     const int per = (op.N + nz - 1) / nz;
     nz = (op.N + per - 1) / per;
-    grow(op.d_fpart, (size_t)nz * npts * nrhs * 3 * sizeof(double2));
-    k_near<<<dim3(npts, nz, groups), 256, 0, s>>>(op.dmesh, geo_of(op), op.k, (const double2*)d_I, nrhs, d_pts, npts,
-                                                  per, op.d_fpart.as<double2>());
-    VIE_CHECK_LAUNCH();
-    const int64_t tot = (int64_t)npts * nrhs * 3;
-    k_near_finish<<<(unsigned)((tot + 127) / 128), 128, 0, s>>>(op.d_fpart.as<double2>(), npts, nrhs, nz,
-                                                                (double2*)d_out);
-    VIE_CHECK_LAUNCH();
+    grow(op.d_fpart, (size_t)nz * pc * nrhs * 3 * sizeof(double2));
+    for (int64_t p0 = 0; p0 < npts; p0 += pc) {
+        const int P = (int)std::min<int64_t>(pc, npts - p0);
+        k_near<<<dim3(P, nz, groups), 256, 0, s>>>(op.dmesh, geo_of(op), op.k, (const double2*)d_I, nrhs,
+                                                   d_pts + 3 * p0, P, per, op.d_fpart.as<double2>());
+        VIE_CHECK_LAUNCH();
+        k_near_finish<<<(P * nrhs * 3 + 127) / 128, 128, 0, s>>>(op.d_fpart.as<double2>(), P, nrhs, nz, p0, npts,
+                                                                 (double2*)d_out);
+        VIE_CHECK_LAUNCH();
+    }
 }
 
 }  // namespace vie
