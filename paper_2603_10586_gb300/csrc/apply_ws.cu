@@ -62,7 +62,6 @@
 // the tensor memory is freed and the CTA exits, the bulk copies that were
 // started and the MMAs that were issued are waited for (with the normal ~1 s
 // limit).  The error word then tells the host.
-#include <cstdlib>
 #include <mutex>
 
 #include "common.h"
@@ -792,18 +791,6 @@ __global__ void __launch_bounds__(128) k_pack_q(const WsClass* __restrict__ cls,
 
 std::once_flag g_ws_attr_once;
 
-// Wait limit of the warp-specialised kernels in clock cycles: ~1 s, or the
-// value of VIE_TEST_WAIT_CYCLES (a test of the timeout path sets it to 0 so
-// that the first wait gives up; the kernels then drain and report).
-long long ws_wait_limit() {
-    const char* e = std::getenv("VIE_TEST_WAIT_CYCLES");
-    if (e && *e) {
-        const long long v = std::atoll(e);
-        return v < 0 ? 0 : v;
-    }
-    return kWaitCycles;
-}
-
 }  // namespace
 
 size_t ws_plane_bytes(const Op& op) {
@@ -864,7 +851,7 @@ static void apply_far_ws(Op& op, const float2* x, int64_t ldx, float2* F, int64_
     }
     if (((uintptr_t)x & 15) || (ldx & 1)) fail(VIE_ERR_INVALID_ARG, "tensor-core apply: x must be 16-byte aligned");
     ws_reserve(op, nrhs);
-    const long long lim = ws_wait_limit();
+    const long long lim = wait_limit(kWaitCycles);
     const int nc = op.ctx->n_sm;
     // the widest tile: 64 columns, or all of them when fewer (a tile never
     // spans two problems' column ranges, so it is no wider than this either)

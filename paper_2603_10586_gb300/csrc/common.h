@@ -431,6 +431,11 @@ void extinction_launch(Op& op, const void* d_I, const double* d_khat, const doub
                        cudaStream_t s);
 void sphere_sum_launch(const void* d_F, const double* d_wt, int npts, int nrhs, double* d_sca, cudaStream_t s);
 
+// limit of a kernel's waits in clock cycles: `normal`, or the value of
+// VIE_TEST_WAIT_CYCLES (a test of the timeout path sets it to 0 so that the first
+// wait gives up; the kernels then drain and report)
+long long wait_limit(long long normal);
+
 // linalg.cu
 void invert_self_blocks(Op& op);   // d_inv64 from d_zself64 (Gauss-Jordan, partial pivoting)
 void convert_c128_to_c64(const void* src, void* dst, int64_t n, cudaStream_t s);

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstdlib>
 #include <limits>
 #include <map>
 #include <numeric>
@@ -21,6 +22,11 @@ void fail(int status, const std::string& msg) { throw Error{status, msg}; }
 double now_s() {
     using namespace std::chrono;
     return duration<double>(steady_clock::now().time_since_epoch()).count();
+}
+
+long long wait_limit(long long normal) {
+    const char* e = std::getenv("VIE_TEST_WAIT_CYCLES");
+    return e && *e ? std::max(0LL, std::atoll(e)) : normal;
 }
 
 static thread_local Ctx* t_alloc_ctx = nullptr;

@@ -24,13 +24,15 @@ namespace {
 // step through memory, on the augmented matrix, took 1.67 ms at np = 108; this
 // takes 0.55 ms.)
 // The row swaps of the pivoting leave the inverse's columns permuted; `perm`
-// undoes that at the end.  The barrier's waits are bounded: status 2.
+// undoes that at the end.  The barrier's waits are bounded (status 2): a grid that gave
+// up is run again as one CTA, which waits for nobody, so a GPU that is kept busy for
+// longer by other work costs time and not the call.
 // ---------------------------------------------------------------------------
 constexpr int kGjThr = 256;
 constexpr size_t kGjSmemMax = 200 * 1024;
 constexpr long long kGjWaitCycles = 2000000000LL;  // ~1 s
 
-__device__ __forceinline__ bool gj_barrier(unsigned* ctr, unsigned target, int* status) {
+__device__ __forceinline__ bool gj_barrier(unsigned* ctr, unsigned target, int* status, long long lim) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -41,7 +43,7 @@ __device__ __forceinline__ bool gj_barrier(unsigned* ctr, unsigned target, int* 
         unsigned v;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-            if (v < target && clock64() - t0 > kGjWaitCycles) {
+            if (v < target && clock64() - t0 >= lim) {
                 atomicExch(status, 2);
                 ok = 0;
                 break;
@@ -54,7 +56,7 @@ __device__ __forceinline__ bool gj_barrier(unsigned* ctr, unsigned target, int* 
 
 __global__ void __launch_bounds__(kGjThr) k_gj_inverse(const double2* __restrict__ A, double2* __restrict__ inv, int np,
                                                        int max_cols, double2* cb, double2* work, int* piv, int* perm,
-                                                       unsigned* ctr, int* status) {
+                                                       unsigned* ctr, int* status, long long lim) {
     extern __shared__ __align__(16) unsigned char gj_smem[];
     const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x;
     const int nc = (np - b + G - 1) / G;  // columns of this CTA: b + c G
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(kGjThr) k_gj_inverse(const double2* __restrict
         if (b + c * G == 0) cb[i] = v;
     }
     unsigned target = G;
-    if (!gj_barrier(ctr, target, status)) return;
+    if (!gj_barrier(ctr, target, status, lim)) return;
     for (int k = 0; k < np; ++k) {
         const double2* col = cb + (size_t)(k & 1) * np;
         double bv = -1.0;
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__(kGjThr) k_gj_inverse(const double2* __restrict
             if (j == k + 1) next[i] = v;
         }
         target += G;
-        if (!gj_barrier(ctr, target, status)) return;
+        if (!gj_barrier(ctr, target, status, lim)) return;
     }
     // column k of the inverse: undo the swaps, last first
     if (b == 0 && tid == 0) {
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kGjThr) k_gj_inverse(const double2* __restrict
         for (int j = 0; j < np; ++j) perm[np + perm[j]] = j;
     }
     target += G;
-    if (!gj_barrier(ctr, target, status)) return;
+    if (!gj_barrier(ctr, target, status, lim)) return;
     for (int e = tid; e < nc * np; e += kGjThr) {
         const int c = e / np, i = e - c * np;
         inv[i + (size_t)__ldcg(perm + np + b + c * G) * np] = M[e];
@@ -282,12 +284,9 @@ __global__ void __launch_bounds__(kGemmThr, 3) type_gemm(const T* __restrict__ M
 
 }  // namespace
 
-void invert_self_blocks(Op& op) {
-    const int np = op.np;
-    cudaStream_t s = op.ctx->stream;
-    op.d_inv64.alloc((size_t)op.T * np * np * sizeof(double2));
-    // two columns per CTA, or as many as one CTA per SM leaves
-    const int G = std::min(op.ctx->n_sm, (np + 1) / 2), max_cols = (np + G - 1) / G;
+// all types' inverses with G CTAs each; returns the kernels' status
+static int gj_run(Op& op, int G, cudaStream_t s) {
+    const int np = op.np, max_cols = (np + G - 1) / G;
     size_t smem = ((size_t)np + 2 * max_cols + (size_t)max_cols * np) * sizeof(double2);
     const bool in_smem = smem <= kGjSmemMax;
     if (!in_smem) smem = 2 * (size_t)max_cols * sizeof(double2);
@@ -303,20 +302,29 @@ void invert_self_blocks(Op& op) {
     int* perm = piv + np;
     int* status = perm + 2 * (size_t)np;
     unsigned* ctr = reinterpret_cast<unsigned*>(status + 1);
+    long long lim = wait_limit(kGjWaitCycles);
     VIE_CUDA(cudaMemsetAsync(status, 0, (1 + op.T) * sizeof(int), s));
     for (int t = 0; t < op.T; ++t) {
         const double2* A = op.d_zself64.as<double2>() + (size_t)t * np * np;
         double2* Inv = op.d_inv64.as<double2>() + (size_t)t * np * np;
         unsigned* c = ctr + t;
         int n = np, mc = max_cols;
-        void* args[] = {&A, &Inv, &n, &mc, &cb, &work, &piv, &perm, &c, &status};
+        void* args[] = {&A, &Inv, &n, &mc, &cb, &work, &piv, &perm, &c, &status, &lim};
         VIE_CUDA(cudaLaunchCooperativeKernel((const void*)k_gj_inverse, dim3(G), dim3(kGjThr), args, smem, s));
         VIE_CHECK_LAUNCH();
     }
     int st = 0;
     VIE_CUDA(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, s));
     VIE_CUDA(cudaStreamSynchronize(s));
-    if (st == 2) fail(VIE_ERR_TIMEOUT, "the inverse of a self block gave up waiting at its barrier");
+    return st;
+}
+
+void invert_self_blocks(Op& op) {
+    cudaStream_t s = op.ctx->stream;
+    op.d_inv64.alloc((size_t)op.T * op.np * op.np * sizeof(double2));
+    // two columns per CTA, or as many as one CTA per SM leaves
+    int st = gj_run(op, std::min(op.ctx->n_sm, (op.np + 1) / 2), s);
+    if (st == 2) st = gj_run(op, 1, s);
     if (st) fail(VIE_ERR_BREAKDOWN, "a meta-atom self block is singular");
 }
 
