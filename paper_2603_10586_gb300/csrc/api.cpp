@@ -124,12 +124,19 @@ using namespace vie;
 
 namespace {
 
+// f is run again once when it was short of memory and the context's operators held
+// optional scratch that could be given back: it starts from its arguments each time
 template <class F>
 int guarded(vie_ctx* ctx, F&& f) {
     cudaGetLastError();  // an earlier failure elsewhere is not this call's error
     AllocScope scope(ctx ? &ctx->c : nullptr);
     try {
-        f();
+        try {
+            f();
+        } catch (const Error& e) {
+            if (!e.memory || !ctx || ctx->c.admitted || !tile_give_back(ctx->c)) throw;
+            f();
+        }
         if (ctx) ctx->c.err.clear();
         return VIE_OK;
     } catch (const Error& e) {
@@ -249,9 +256,10 @@ const char* vie_last_error(vie_ctx* ctx) { return ctx ? ctx->c.err.c_str() : "no
 int vie_assemble(vie_ctx* ctx, const vie_geometry* g, double wavelength, vie_op** out) {
     if (!ctx || !g || !out) return VIE_ERR_INVALID_ARG;
     *out = nullptr;
-    auto op = std::make_unique<vie_op>();
+    std::unique_ptr<vie_op> op;
     int st = guarded(ctx, [&] {
         set_device(ctx->c);
+        op = std::make_unique<vie_op>();
         Op& o = op->o;
         o.ctx = &ctx->c;
         double t0 = now_s();

@@ -474,22 +474,59 @@ bool tile_pays(const Op& op, int nrhs) {
     return op.share_mean * nrhs >= least || few;
 }
 
+Op::~Op() {
+    if (!ctx) return;
+    auto& v = ctx->tile_ops;
+    v.erase(std::remove(v.begin(), v.end(), this), v.end());
+}
+
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
     const size_t rp = pass_cols(op, nrhs, elem);
     const size_t np = (size_t)std::max<int64_t>(op.part_total, 1) * rp * elem;
     const size_t nt = (size_t)std::max<int64_t>(op.ct_total, 1) * rp * elem;
-    if (op.d_part.bytes >= np && op.d_ct.bytes >= nt) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     VIE_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (cap != cudaStreamCaptureStatusNone) return false;
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    if (op.d_part.bytes >= np && op.d_ct.bytes >= nt) {
+        op.tile_pinned |= capturing;
+        return true;
+    }
+    if (capturing || (op.tile_oom && np + nt >= op.tile_oom)) return false;
+    auto& v = op.ctx->tile_ops;
+    if (std::find(v.begin(), v.end(), &op) == v.end()) v.push_back(&op);
     try {
+        if (np + nt > ((size_t)256 << 20) && !op.ctx->admitted) {  // leave 1 GiB to the solver, as ws_pack does
+            size_t free_b = 0, total_b = 0;
+            VIE_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            if (np + nt + ((size_t)1 << 30) > free_b + op.d_part.bytes + op.d_ct.bytes)
+                fail(VIE_ERR_OOM, "no room for the register tiles' scratch");
+        }
         if (op.d_part.bytes < np) op.d_part.alloc(np);
         if (op.d_ct.bytes < nt) op.d_ct.alloc(nt);
     } catch (const Error& e) {
-        if (e.status != VIE_ERR_OOM || op.ctx->admitted) throw;
+        if (e.status != VIE_ERR_OOM) throw;
+        if (!op.tile_pinned) {
+            op.d_part.release();
+            op.d_ct.release();
+        }
+        if (op.ctx->admitted) throw;
+        op.tile_oom = np + nt;
         return false;
     }
     return true;
+}
+
+bool tile_give_back(Ctx& c) {
+    bool any = false;
+    for (Op* o : c.tile_ops) {
+        const size_t held = o->d_part.bytes + o->d_ct.bytes;
+        if (o->tile_pinned || held == 0) continue;
+        o->d_part.release();
+        o->d_ct.release();
+        o->tile_oom = o->tile_oom ? std::min(o->tile_oom, held) : held;
+        any = true;
+    }
+    return any;
 }
 
 template <class TF, class TX, class TO>

@@ -26,6 +26,7 @@ using cd = std::complex<double>;
 struct Error {
     int status;
     std::string msg;
+    bool memory = false;  // device memory was short (the context's cap, or the GPU's)
 };
 
 [[noreturn]] void fail(int status, const std::string& msg);
@@ -217,6 +218,13 @@ struct Op {
     DevBuf d_cmem, d_c1_items, d_c2_items, d_cseg, d_ctoff, d_pbase, d_ct, d_part;
     DevBuf d_c1_long, d_c2_long;  // the items, longest first (tile_long)
     bool tile_long = false;
+    // d_ct and d_part are optional (the per-block kernels do without) and large: what
+    // could not be had is not asked for again (tile_oom: its bytes, 0 none; until the next
+    // compression), and they are given back when a call is short of memory, unless a
+    // graph that the caller captured holds their addresses
+    size_t tile_oom = 0;
+    bool tile_pinned = false;
+    ~Op();
     static constexpr size_t kTilePass = (size_t)2 << 30;  // partial products of one pass (or sixteen columns')
     int n_c1_items = 0, n_c2_items = 0, tile_seg = 512;
     int n_cseg = 0, tile_group = 1;  // blocks with several segments, members of the largest group
@@ -292,6 +300,7 @@ struct Ctx {
     std::atomic<int64_t> allocated{0}, peak{0};
     std::atomic<int64_t> cap{0};
     bool admitted = false;  // a server's slot: a request that meets the cap is run again with more
+    std::vector<Op*> tile_ops;  // operators that hold register-tile scratch
     // joined operators of recent vie_solve_batch calls (block-diagonal unions of
     // their problems), reused while the same operators with the same factors
     // come again; declared last so that they are freed first
@@ -491,6 +500,9 @@ void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t
 // depend on the cap it first met.
 bool tile_pays(const Op& op, int nrhs);
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s);
+// gives back the scratch of the context's operators (not what a caller's graph holds), for a
+// call that is short of memory; false when there was none
+bool tile_give_back(Ctx& c);
 template <class TF, class TX, class TO>
 void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nrhs, cudaStream_t s, int first = 0,
                     int count = -1);  // columns [first, first + count) of the call (-1: all)

@@ -55,8 +55,8 @@ void DevBuf::alloc(size_t b) {
         const int64_t now = c->allocated.fetch_add((int64_t)b) + (int64_t)b;
         if (cap > 0 && now > cap) {
             c->allocated.fetch_sub((int64_t)b);
-            fail(VIE_ERR_OOM, "allocation of " + std::to_string(b) + " bytes would exceed the context's cap of " +
-                                  std::to_string(cap) + " bytes");
+            throw Error{VIE_ERR_OOM, "allocation of " + std::to_string(b) + " bytes would exceed the context's cap of " +
+                                         std::to_string(cap) + " bytes", true};
         }
     }
     // (the null stream names no stream to free on: such a buffer is not pooled)
@@ -73,7 +73,8 @@ void DevBuf::alloc(size_t b) {
         p = nullptr;
         if (c) c->allocated.fetch_sub((int64_t)b);
         cudaGetLastError();
-        fail(VIE_ERR_OOM, "cudaMalloc of " + std::to_string(b) + " bytes failed: " + cudaGetErrorString(e));
+        throw Error{VIE_ERR_OOM, "cudaMalloc of " + std::to_string(b) + " bytes failed: " + cudaGetErrorString(e),
+                    e == cudaErrorMemoryAllocation};
     }
     bytes = b;
     owner = c;
@@ -566,6 +567,8 @@ void build_apply_lists(Op& op) {
         upload(op.d_ctoff, ctoff);
         op.d_part.release();  // sized on first use (tile_reserve)
         op.d_ct.release();
+        op.tile_oom = 0;
+        op.tile_pinned = false;
     }
 }
 

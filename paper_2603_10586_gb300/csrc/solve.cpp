@@ -178,7 +178,10 @@ struct Gmres {
         VIE_CUDA(cudaMallocHost(reinterpret_cast<void**>(&h_pinned), (KR_NCTR + nrhs) * sizeof(int)));
     }
 
+    const bool tile_pinned = op.tile_pinned;  // (the graphs captured here go with this object)
+
     ~Gmres() {
+        op.tile_pinned = tile_pinned;
         for (auto& kv : graphs)
             if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
         if (s_body) cudaStreamDestroy(s_body);
