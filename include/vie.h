@@ -406,8 +406,9 @@ int vie_lpt_assign(const double* w, int64_t n, int n_proc, int* owner, double* l
  * the budget; admitted requests run concurrently, each on its own CUDA stream.
  * A request's allocations are capped at its admitted footprint; one that
  * reaches the cap goes back to the head of the queue with twice the footprint
- * (at most the budget) and runs again when that much is free; one that fails
- * with the whole budget returns VIE_ERR_ADMISSION. */
+ * (at most the budget) and runs again when that much is free; with the whole
+ * budget it does without optional scratch, and one that fails even so returns
+ * VIE_ERR_ADMISSION. */
 typedef struct vie_serve_opts {
     int max_inflight;          /* concurrent requests (slots) */
     size_t hbm_budget;         /* bytes for all in-flight requests (0 = context budget) */

@@ -156,10 +156,11 @@ vie_ctx* ctx_of(vie_op* op) { return op ? static_cast<vie_ctx*>(op->o.ctx->owner
 }  // namespace
 
 // server use: the cap of a slot context is the footprint its request was
-// admitted with; the peak shows what the request really held
-void ctx_set_cap(vie_ctx* ctx, int64_t cap) {
+// admitted with (last: the whole budget, there will be no more); the peak shows what
+// the request really held
+void ctx_set_cap(vie_ctx* ctx, int64_t cap, bool last) {
     ctx->c.cap = cap;
-    ctx->c.admitted = cap > 0;
+    ctx->c.admitted = cap > 0 && !last;
     ctx->c.peak = ctx->c.allocated.load();
 }
 int64_t ctx_peak(vie_ctx* ctx) { return ctx->c.peak.load(); }

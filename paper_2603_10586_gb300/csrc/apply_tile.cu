@@ -451,16 +451,16 @@ __global__ void __launch_bounds__(128) k_tile_sum(const int4* __restrict__ items
     store(F + (int64_t)a * np + row + (int64_t)c * ldf, acc);
 }
 
+}  // namespace
+
 // right-hand sides per pass: their partial products stay within kTilePass bytes, or
 // sixteen columns' (few columns leave tiles empty: 11 columns of the 27 x 27 graded
 // array of 4^3 cubes in double-float, one at a time, took 59 ms).  At most 1024,
 // which Cols::member needs.
-int pass_cols(const Op& op, int nrhs, size_t elem) {
-    const size_t per = (size_t)std::max<int64_t>(op.part_total, 1) * elem;
+int tile_pass_cols(int64_t part_total, int nrhs, size_t elem) {
+    const size_t per = (size_t)std::max<int64_t>(part_total, 1) * elem;
     return (int)std::min<size_t>(std::min(nrhs, 1024), std::max<size_t>(16, Op::kTilePass / per));
 }
-
-}  // namespace
 
 // The tile kernels read a factor once per group of columns; the per-block kernels
 // once per right-hand side or four of them, but without partial products.  Without
@@ -481,7 +481,7 @@ Op::~Op() {
 }
 
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
-    const size_t rp = pass_cols(op, nrhs, elem);
+    const size_t rp = tile_pass_cols(op.part_total, nrhs, elem);
     const size_t np = (size_t)std::max<int64_t>(op.part_total, 1) * rp * elem;
     const size_t nt = (size_t)std::max<int64_t>(op.ct_total, 1) * rp * elem;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -533,7 +533,7 @@ template <class TF, class TX, class TO>
 void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nrhs, cudaStream_t s, int first,
                     int count) {
     const int last = count < 0 ? nrhs : first + count;
-    const int rp = pass_cols(op, last - first, sizeof(TX));
+    const int rp = tile_pass_cols(op.part_total, last - first, sizeof(TX));
     TX* t = op.d_ct.as<TX>();
     TX* P = op.d_part.as<TX>();
     constexpr size_t smem1 = smem_bytes<TF, TX>(1), smem2 = smem_bytes<TF, TX>(2);

@@ -299,7 +299,9 @@ struct Ctx {
     // (0: none) above which an allocation is refused with VIE_ERR_OOM
     std::atomic<int64_t> allocated{0}, peak{0};
     std::atomic<int64_t> cap{0};
-    bool admitted = false;  // a server's slot: a request that meets the cap is run again with more
+    // a server's slot whose request is run again with more when it meets the cap, so that its
+    // result does not depend on the cap (at the whole budget it makes do without scratch)
+    bool admitted = false;
     std::vector<Op*> tile_ops;  // operators that hold register-tile scratch
     // joined operators of recent vie_solve_batch calls (block-diagonal unions of
     // their problems), reused while the same operators with the same factors
@@ -495,10 +497,10 @@ void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t
 // apply_tile.cu: far apply by register tiles over classes of blocks that share
 // their factors.  tile_reserve: its scratch for nrhs columns of `elem`-byte
 // vector elements; false when the memory is not there (or would have to be allocated
-// while `s` is capturing), and the per-block kernels run instead.  In a server's slot
-// VIE_ERR_OOM: the request runs again with a larger footprint, and its result does not
-// depend on the cap it first met.
+// while `s` is capturing), and the per-block kernels run instead; VIE_ERR_OOM in a
+// server's slot whose request can still be given more (Ctx::admitted).
 bool tile_pays(const Op& op, int nrhs);
+int tile_pass_cols(int64_t part_total, int nrhs, size_t elem);  // right-hand sides per pass
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s);
 // gives back the scratch of the context's operators (not what a caller's graph holds), for a
 // call that is short of memory; false when there was none

@@ -13,8 +13,10 @@
 // request was promised: the allocation fails with VIE_ERR_OOM on the host,
 // and the request goes back to the head of the queue with twice the
 // footprint (at most the whole budget), to run again once that much is free.
-// A request that fails this way with the whole budget is rejected.
+// With the whole budget a request that lacks only the register tiles' scratch runs
+// without it; one that fails even so is rejected.
 #include <chrono>
+#include <cmath>
 #include <cstdlib>
 #include <condition_variable>
 #include <cstring>
@@ -27,7 +29,7 @@
 #include "common.h"
 
 // slot-context hooks of the library (api.cpp)
-void ctx_set_cap(vie_ctx* ctx, int64_t cap);
+void ctx_set_cap(vie_ctx* ctx, int64_t cap, bool last);
 int64_t ctx_peak(vie_ctx* ctx);
 
 namespace {
@@ -50,7 +52,16 @@ struct Done {
     bool ready = false;
 };
 
-int64_t model_footprint(const Pending& p, int restart) {
+// What a request is admitted with (its least, `need`, must fit the budget) and what it
+// is expected to hold in its solve, where the Krylov bases of all columns, the solver's
+// vectors and the register tiles' scratch count: it is given that much from the start when the
+// budget has it, since a request that meets its cap begins again from its assembly.
+struct Footprint {
+    int64_t need, want;
+};
+
+Footprint model_footprint(const Pending& p, const vie_solve_opts& o) {
+    const int restart = o.restart;
     const int nv = p.nv[0];
     const int np = 3 * (nv + 1) * nv * nv;
     const int64_t n = (int64_t)p.n_atoms * np;
@@ -58,17 +69,34 @@ int64_t model_footprint(const Pending& p, int restart) {
     while ((1LL << (2 * levels)) < p.n_atoms) ++levels;
     // rank model: ~64 per far block row/column per level (measured ranks at
     // tolerance 1e-4 are of this order for sub-wavelength atoms)
-    int64_t factor_entries = 2 * n * 64 * std::max(1, levels - 1);
+    const int64_t factor_entries = 2 * n * 64 * std::max(1, levels - 1);
     int64_t b = vie_footprint_bytes(n, np, p.nrhs, restart, factor_entries);
     // compression workspace: the largest batch of formed blocks
     int64_t big = std::min<int64_t>(n, (int64_t)16 * np);
     b += std::min<int64_t>(big * big * 8 * 4, (int64_t)8 << 30);
+    // far blocks per target atom, mean over a full grid of 2^levels boxes per side
+    // (28 x 28 atoms: 81, counted 77; 48 x 48: 107 and 95; 500 on a spiral: 81 and 69)
+    double per_atom = 0;
+    for (int l = 2; l <= levels; ++l)
+        per_atom += std::pow(6.0 - 8.0 / (1 << l), 2) - std::pow(3.0 - 2.0 / (1 << l), 2);
+    if (levels > 0) per_atom += std::pow(3.0 - 2.0 / (1 << levels), 2) - 1.0;
+    // partial products, and t, whose segments were counted at 0.4 to 0.5 of them on atoms of
+    // 108 and 240 unknowns and at 0.9 to 1.0 on atoms of 36
+    const double part = per_atom * (double)n, ct = part * std::min(1.0, std::max(0.5, 36.0 / np));
+    const int64_t cols = vie::tile_pass_cols((int64_t)part, p.nrhs, sizeof(double2));
+    // (BiCGStab keeps no basis)
+    const int64_t basis = o.method == 1 ? 0 : std::min(restart > 0 ? restart : 60, 512) + 1;
+    const double solve = 16.0 * ((double)p.nrhs * ((double)(basis + 12) * n + ct) + (part + ct) * (double)cols);
+    int64_t w = 8 * factor_entries + 3 * (int64_t)np * np * 48 + (int64_t)solve;
     // a test of the back-off path scales the model down (VIE_TEST_FOOTPRINT_SCALE)
     if (const char* e = std::getenv("VIE_TEST_FOOTPRINT_SCALE")) {
         const double f = std::atof(e);
-        if (f > 0) b = std::max<int64_t>(1 << 20, (int64_t)(b * f));
+        if (f > 0) {
+            b = std::max<int64_t>(1 << 20, (int64_t)(b * f));
+            w = (int64_t)(w * f);
+        }
     }
-    return b;
+    return {b, std::max(b, w)};
 }
 
 }  // namespace
@@ -114,7 +142,7 @@ struct vie_server {
             res.footprint_bytes = p.footprint;
             vie_geometry g{p.n_atoms, p.centres.data(), p.types.data(), p.n_types, p.sides.data(), p.nv.data(),
                            p.eps.data()};
-            ctx_set_cap(ctx, p.footprint);
+            ctx_set_cap(ctx, p.footprint, p.footprint >= budget);
             vie_op* op = nullptr;
             int st = vie_assemble(ctx, &g, p.wavelength, &op);
             if (st == VIE_OK) st = vie_compress(op, opts.tol > 0 ? opts.tol : 1e-4, VIE_C64);
@@ -206,10 +234,11 @@ int vie_submit(vie_server* s, const vie_request* req, uint64_t* ticket) {
     p.eps.assign(g.eps, g.eps + 2 * g.n_types);
     p.khat.assign(req->inc.khat, req->inc.khat + 3 * req->nrhs);
     p.pol.assign(req->inc.pol, req->inc.pol + 6 * req->nrhs);
-    p.footprint = model_footprint(p, s->opts.solve.restart);
+    const Footprint f = model_footprint(p, s->opts.solve);
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->stopping) return VIE_ERR_STATE;
-    if (p.footprint > s->budget) return VIE_ERR_ADMISSION;
+    if (f.need > s->budget) return VIE_ERR_ADMISSION;
+    p.footprint = std::min(f.want, s->budget);
     p.ticket = s->next_ticket++;
     p.t_submit = s->clock_s();
     *ticket = p.ticket;
