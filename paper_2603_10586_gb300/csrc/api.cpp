@@ -164,6 +164,7 @@ void ctx_set_cap(vie_ctx* ctx, int64_t cap, bool last) {
     ctx->c.peak = ctx->c.allocated.load();
 }
 int64_t ctx_peak(vie_ctx* ctx) { return ctx->c.peak.load(); }
+void ctx_trim(vie_ctx* ctx) { ctx->c.pool_trim(); }
 
 namespace {
 
@@ -204,18 +205,6 @@ int vie_create(vie_ctx** out, const vie_ctx_opts* opts) {
         VIE_CUDA(cudaGetDeviceProperties(&prop, c.device));
         c.n_sm = prop.multiProcessorCount;
         VIE_CUDA(cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking));
-        cudaMemPoolProps pp = {};
-        pp.allocType = cudaMemAllocationTypePinned;
-        pp.handleTypes = cudaMemHandleTypeNone;
-        pp.location.type = cudaMemLocationTypeDevice;
-        pp.location.id = c.device;
-        if (cudaMemPoolCreate(&c.pool, &pp) == cudaSuccess) {
-            uint64_t keep = Ctx::kPoolKeep;
-            cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        } else {  // ordinary allocations instead
-            c.pool = nullptr;
-            cudaGetLastError();
-        }
         VIE_BLAS(cublasCreate(&c.blas));
         VIE_BLAS(cublasSetStream(c.blas, c.stream));
         size_t fr = 0, tot = 0;
@@ -223,6 +212,7 @@ int vie_create(vie_ctx** out, const vie_ctx_opts* opts) {
         size_t reserve = (size_t)4 << 30;
         c.budget = (opts && opts->hbm_budget) ? opts->hbm_budget : (fr > 2 * reserve ? fr - reserve : fr / 2);
         c.cap = (opts && opts->hbm_budget) ? (int64_t)opts->hbm_budget : 0;
+        c.pool_open();  // last: from here on the context is closed by free_ctx
     });
     if (st != VIE_OK) {
         // keep the message readable through a stub context
@@ -237,11 +227,8 @@ int vie_create(vie_ctx** out, const vie_ctx_opts* opts) {
 static void free_ctx(vie_ctx* ctx) {
     cudaSetDevice(ctx->c.device);
     if (ctx->c.blas) cublasDestroy(ctx->c.blas);
-    if (ctx->c.pool) {
-        ctx->c.unions.clear();  // (their buffers are not pooled; freed before the stream)
-        cudaStreamSynchronize(ctx->c.stream);
-        cudaMemPoolDestroy(ctx->c.pool);
-    }
+    ctx->c.unions.clear();  // (their buffers are not pooled; freed before the stream)
+    ctx->c.pool_close();
     if (ctx->c.stream) cudaStreamDestroy(ctx->c.stream);
     delete ctx;
 }

@@ -289,6 +289,11 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     cudaMemPool_t pool = nullptr;  // TmpBufs; keeps at most kPoolKeep bytes between calls
     static constexpr size_t kPoolKeep = (size_t)256 << 20;
+    static constexpr int64_t kPoolChunk = (int64_t)32 << 20;  // the driver's step of a pool's memory
+    void pool_open();              // creates the pool (none: ordinary allocations instead)
+    void pool_close();
+    void pool_trim();              // waits for `stream` and gives back what the pool keeps
+    int64_t pool_kept() const;     // bytes it keeps beyond its buffers, but for one chunk
     cublasHandle_t blas = nullptr;
     std::string err;
     size_t budget = 0;

@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <limits>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <queue>
 #include <unordered_map>
@@ -46,13 +47,68 @@ TmpScope::~TmpScope() {
     t_tmp_on = prev_on;
 }
 
+// The open pools of the process: an allocation that the GPU has no room for takes back
+// what any of them keeps, not only its own context's.
+static std::mutex g_pools_mu;
+static std::vector<Ctx*> g_pools;
+
+void Ctx::pool_open() {
+    cudaMemPoolProps pp = {};
+    pp.allocType = cudaMemAllocationTypePinned;
+    pp.handleTypes = cudaMemHandleTypeNone;
+    pp.location.type = cudaMemLocationTypeDevice;
+    pp.location.id = device;
+    if (cudaMemPoolCreate(&pool, &pp) != cudaSuccess) {
+        pool = nullptr;
+        cudaGetLastError();
+        return;
+    }
+    uint64_t keep = kPoolKeep;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    std::lock_guard<std::mutex> lk(g_pools_mu);
+    g_pools.push_back(this);
+}
+
+void Ctx::pool_close() {
+    if (!pool) return;
+    {
+        std::lock_guard<std::mutex> lk(g_pools_mu);
+        g_pools.erase(std::find(g_pools.begin(), g_pools.end(), this));
+    }
+    cudaStreamSynchronize(stream);
+    cudaMemPoolDestroy(pool);
+    pool = nullptr;
+}
+
+void Ctx::pool_trim() {
+    if (!pool) return;
+    cudaStreamSynchronize(stream);
+    cudaMemPoolTrimTo(pool, 0);
+}
+
+int64_t Ctx::pool_kept() const {
+    uint64_t reserved = 0, used = 0;
+    if (!pool || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+        return 0;
+    return std::max<int64_t>(0, (int64_t)reserved - (int64_t)used - kPoolChunk);
+}
+
 void DevBuf::alloc(size_t b) {
     release();
     if (b == 0) b = 1;
     Ctx* c = t_alloc_ctx;
+    int64_t kept = 0;  // what the pool keeps counts against a cap
     if (c) {
         const int64_t cap = c->cap.load();
         const int64_t now = c->allocated.fetch_add((int64_t)b) + (int64_t)b;
+        if (cap > 0) {
+            kept = c->pool_kept();
+            if (kept > 0 && now + kept > cap) {
+                c->pool_trim();
+                kept = c->pool_kept();
+            }
+        }
         if (cap > 0 && now > cap) {
             c->allocated.fetch_sub((int64_t)b);
             throw Error{VIE_ERR_OOM, "allocation of " + std::to_string(b) + " bytes would exceed the context's cap of " +
@@ -62,10 +118,14 @@ void DevBuf::alloc(size_t b) {
     // (the null stream names no stream to free on: such a buffer is not pooled)
     const bool pooled = tmp && t_tmp_on && t_tmp_stream && c && c->pool && b <= TmpBuf::kPoolMax;
     cudaError_t e = pooled ? cudaMallocFromPoolAsync(&p, b, c->pool, t_tmp_stream) : cudaMalloc(&p, b);
-    if (e == cudaErrorMemoryAllocation && c && c->pool) {  // give back what the pool keeps and try again
+    if (e == cudaErrorMemoryAllocation && c) {  // give back what the pools keep and try again
         cudaGetLastError();
         cudaStreamSynchronize(pooled ? t_tmp_stream : c->stream);
-        cudaMemPoolTrimTo(c->pool, 0);
+        {
+            std::lock_guard<std::mutex> lk(g_pools_mu);
+            for (Ctx* o : g_pools)
+                if (o->device == c->device) cudaMemPoolTrimTo(o->pool, 0);
+        }
         e = pooled ? cudaMallocFromPoolAsync(&p, b, c->pool, t_tmp_stream) : cudaMalloc(&p, b);
     }
     if (e == cudaSuccess && pooled) stream = t_tmp_stream;
@@ -79,7 +139,7 @@ void DevBuf::alloc(size_t b) {
     bytes = b;
     owner = c;
     if (c) {
-        int64_t pk = c->peak.load(), cur = c->allocated.load();
+        int64_t pk = c->peak.load(), cur = c->allocated.load() + kept;
         while (cur > pk && !c->peak.compare_exchange_weak(pk, cur)) {
         }
     }

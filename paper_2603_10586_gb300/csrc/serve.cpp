@@ -9,8 +9,8 @@
 // alone is rejected (VIE_ERR_ADMISSION).  Every wait is bounded.
 //
 // The slot's context refuses allocations beyond the footprint its request
-// was admitted with, so an under-estimate cannot take memory that another
-// request was promised: the allocation fails with VIE_ERR_OOM on the host,
+// was admitted with (whole chunks that its pool of temporaries keeps count), so
+// an under-estimate cannot take memory that another request was promised: the allocation fails with VIE_ERR_OOM on the host,
 // and the request goes back to the head of the queue with twice the
 // footprint (at most the whole budget), to run again once that much is free.
 // With the whole budget a request that lacks only the register tiles' scratch runs
@@ -31,6 +31,7 @@
 // slot-context hooks of the library (api.cpp)
 void ctx_set_cap(vie_ctx* ctx, int64_t cap, bool last);
 int64_t ctx_peak(vie_ctx* ctx);
+void ctx_trim(vie_ctx* ctx);
 
 namespace {
 
@@ -158,6 +159,7 @@ struct vie_server {
             }
             if (op) vie_op_destroy(op);
             res.peak_bytes = ctx_peak(ctx);
+            ctx_trim(ctx);  // the footprint goes back whole
             if (st == VIE_ERR_OOM) {
                 std::free(res.I);
                 res.I = nullptr;
