@@ -115,7 +115,7 @@ void op_reserve(Op& op, int nrhs, int precision, cudaStream_t s) {
         for (int k = 1; k <= nrhs; ++k) {
             const int v = far_variant(op, inner, k);
             if (v == VIE_VAR_SIMT_SHARED) cols = std::max(cols, 1);
-            else if (v >= VIE_VAR_SIMT_R2 && v <= VIE_VAR_SIMT_R8 && tile_pays(op, k)) cols = k;
+            else if (v >= VIE_VAR_SIMT_R2 && v <= VIE_VAR_SIMT_R8 && far_tiled(op, inner, k)) cols = k;
         }
         if (cols > 0) tile_reserve(op, cols, sizeof(float2), s);
     }

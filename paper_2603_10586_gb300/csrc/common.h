@@ -264,6 +264,9 @@ struct Op {
     // far-apply variant per (precision, log2 of the right-hand-side count),
     // chosen by the autotuner or set by the caller
     std::map<std::pair<int, int>, int> variant;
+    // and, where the autotuner chose one of SIMT_R2..R8, its form as measured: register
+    // tiles or per-block kernels (otherwise tile_pays decides)
+    std::map<std::pair<int, int>, bool> tiled;
     // scratch
     DevBuf d_t, d_F;
     DevBuf d_xs;  // float64 vectors split into float32 head + tail (double-float apply)
@@ -505,6 +508,7 @@ void apply_far_umma_ws2(Op& op, const float2* x, int64_t ldx, float2* F, int64_t
 // while `s` is capturing), and the per-block kernels run instead; VIE_ERR_OOM in a
 // server's slot whose request can still be given more (Ctx::admitted).
 bool tile_pays(const Op& op, int nrhs);
+bool far_tiled(const Op& op, int precision, int nrhs);  // tile_pays, or the autotuner's choice
 int tile_pass_cols(int64_t part_total, int nrhs, size_t elem);  // right-hand sides per pass
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s);
 // gives back the scratch of the context's operators (not what a caller's graph holds), for a

@@ -46,8 +46,9 @@ int default_variant(const Op& op, int precision, int nrhs) {
 // the variants that read a factor once per group of right-hand sides: the
 // register tiles take all columns (copies x right-hand sides) of a factor
 // together where that pays, in one summation order for the three group sizes
-void far_grouped(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, int nr, cudaStream_t s) {
-    if (tile_pays(op, nrhs) && tile_reserve(op, nrhs, sizeof(float2), s))
+void far_grouped(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, int nr, int precision,
+                 cudaStream_t s) {
+    if (far_tiled(op, precision, nrhs) && tile_reserve(op, nrhs, sizeof(float2), s))
         apply_far_tile<float2, float2, float2>(op, x, ldx, F, ldf, nrhs, s);
     else
         apply_far_simt32(op, x, ldx, F, ldf, nrhs, nr, s);
@@ -60,12 +61,17 @@ int far_variant(const Op& op, int precision, int nrhs) {
     return it != op.variant.end() ? it->second : default_variant(op, precision, nrhs);
 }
 
+bool far_tiled(const Op& op, int precision, int nrhs) {
+    const auto it = op.tiled.find({precision, bucket(nrhs)});
+    return it != op.tiled.end() ? it->second : tile_pays(op, nrhs);
+}
+
 void far32(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, int precision, cudaStream_t s) {
     switch (far_variant(op, precision, nrhs)) {
         case VIE_VAR_SIMT_R1: apply_far_simt32(op, x, ldx, F, ldf, nrhs, 1, s); break;
-        case VIE_VAR_SIMT_R2: far_grouped(op, x, ldx, F, ldf, nrhs, 2, s); break;
-        case VIE_VAR_SIMT_R4: far_grouped(op, x, ldx, F, ldf, nrhs, 4, s); break;
-        case VIE_VAR_SIMT_R8: far_grouped(op, x, ldx, F, ldf, nrhs, 8, s); break;
+        case VIE_VAR_SIMT_R2: far_grouped(op, x, ldx, F, ldf, nrhs, 2, precision, s); break;
+        case VIE_VAR_SIMT_R4: far_grouped(op, x, ldx, F, ldf, nrhs, 4, precision, s); break;
+        case VIE_VAR_SIMT_R8: far_grouped(op, x, ldx, F, ldf, nrhs, 8, precision, s); break;
         case VIE_VAR_MMA_BF16X3: apply_far_bf16x3(op, x, ldx, F, ldf, nrhs, s); break;
         case VIE_VAR_TCGEN05_BF16X3: apply_far_umma(op, x, ldx, F, ldf, nrhs, s); break;
         case VIE_VAR_TCGEN05_PACKED_BF16X3: apply_far_umma_packed(op, x, ldx, F, ldf, nrhs, s); break;
@@ -115,32 +121,48 @@ int tune_far(Op& op, int precision, int nrhs, cudaStream_t s, std::vector<int>& 
     } guard{op, op.colr};
     op.colr = nullptr;
     const auto key = std::make_pair(precision, bucket(nrhs));
-    const auto saved = op.variant.find(key) != op.variant.end() ? op.variant[key] : 0;
+    const auto had_variant = op.variant.find(key) != op.variant.end() ? op.variant[key] : 0;
+    const auto had_form = op.tiled;
     int best = 0;
+    bool best_form = false;
     double best_ms = 1e300;
+    auto time_one = [&] {
+        far32(op, x.as<float2>(), n, F.as<float2>(), n, nrhs, precision, s);  // warm-up
+        double t = 1e300;
+        for (int r = 0; r < 3; ++r) {
+            VIE_CUDA(cudaEventRecord(e0, s));
+            far32(op, x.as<float2>(), n, F.as<float2>(), n, nrhs, precision, s);
+            VIE_CUDA(cudaEventRecord(e1, s));
+            VIE_CUDA(cudaEventSynchronize(e1));
+            float m = 0.f;
+            VIE_CUDA(cudaEventElapsedTime(&m, e0, e1));
+            t = std::min(t, (double)m);
+        }
+        return t;
+    };
     try {
         for (int v : cand) {
             op.variant[key] = v;
-            far32(op, x.as<float2>(), n, F.as<float2>(), n, nrhs, precision, s);  // warm-up
+            // R2, R4, R8 as per-block kernels; the register tiles, one kernel for the
+            // three, beside R4
+            const bool grouped = v >= VIE_VAR_SIMT_R2 && v <= VIE_VAR_SIMT_R8;
             double t = 1e300;
-            for (int r = 0; r < 3; ++r) {
-                VIE_CUDA(cudaEventRecord(e0, s));
-                far32(op, x.as<float2>(), n, F.as<float2>(), n, nrhs, precision, s);
-                VIE_CUDA(cudaEventRecord(e1, s));
-                VIE_CUDA(cudaEventSynchronize(e1));
-                float m = 0.f;
-                VIE_CUDA(cudaEventElapsedTime(&m, e0, e1));
-                t = std::min(t, (double)m);
+            for (int form = 0; form < (v == VIE_VAR_SIMT_R4 ? 2 : 1); ++form) {
+                if (grouped) op.tiled[key] = form == 1;
+                const double tf = time_one();
+                t = std::min(t, tf);
+                if (tf < best_ms) {
+                    best_ms = tf;
+                    best = v;
+                    best_form = form == 1;
+                }
             }
             ms.push_back(t);
-            if (t < best_ms) {
-                best_ms = t;
-                best = v;
-            }
         }
     } catch (...) {
-        if (saved) op.variant[key] = saved;
+        if (had_variant) op.variant[key] = had_variant;
         else op.variant.erase(key);
+        op.tiled = had_form;
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         throw;
@@ -148,6 +170,8 @@ int tune_far(Op& op, int precision, int nrhs, cudaStream_t s, std::vector<int>& 
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     op.variant[key] = best;
+    if (best >= VIE_VAR_SIMT_R2 && best <= VIE_VAR_SIMT_R8) op.tiled[key] = best_form;
+    else op.tiled.erase(key);
     return best;
 }
 
@@ -160,6 +184,7 @@ int tune_entry(Op& op, int precision, int nrhs, int force, vie_tune_result* res,
         if (op.fprec != VIE_C64) fail(VIE_ERR_INVALID_ARG, "vie_tune: needs VIE_C64 factors");
         if (nrhs < 1 || nrhs > 1024) fail(VIE_ERR_INVALID_ARG, "vie_tune: 1 to 1024 right-hand sides");
         op.variant[{precision, bucket(nrhs)}] = force;
+        op.tiled.erase({precision, bucket(nrhs)});
         v = force;
     } else {
         v = tune_far(op, precision, nrhs, s, cand, ms);
