@@ -94,19 +94,21 @@ enum vie_variant {
                                side when the operator has translated copies) */,
     VIE_VAR_TCGEN05_WS_BF16X3 = 9 /* the factors split once into bf16 planes, held once per factor
                                      storage (translated copies share them), in a warp-specialised
-                                     persistent kernel (one CTA per SM): a warp moves the A planes by bulk
-                                     TMA into a ring of 4 or 5 stages, up to four warp pairs gather and split B into two stacked plane
-                                     sets, a warp issues four wide MMAs per K step (each A plane read
-                                     once), four warps drain two tensor-memory accumulator buffers; equal
-                                     to 7 to float32 rounding (default for 8 to 32 right-hand sides on
-                                     atoms of at most 128 unknowns; runs as 10 above 32 right-hand sides, as
-                                     6 when the planes do not fit) */,
+                                     persistent kernel (one CTA per SM): a warp moves the A planes by
+                                     bulk TMA into a ring of 4 or 5 stages, four warp pairs gather and
+                                     split B into two stacked plane sets, a warp issues four wide MMAs
+                                     per K step (each A plane read once), four warps drain two
+                                     tensor-memory accumulator buffers; equal to 7 to float32 rounding
+                                     (default for 8 to 32 right-hand sides on atoms of at most 128
+                                     unknowns, and on larger atoms where the SMs' lists of 10 would be
+                                     unbalanced; runs as 10 above 32 right-hand sides, as 6 when the
+                                     planes do not fit) */,
     VIE_VAR_TCGEN05_WS2_BF16X3 = 10 /* 9 with two 128-row tiles of factor rows sharing each B tile (the
                                        two row tiles of a target atom, or two consecutive row tiles of
-                                       a source group), 16 K values per stage: the B operand is gathered
-                                       and split once for twice the rows; equal to 9 to float32
-                                       rounding (default for 8 right-hand sides or more otherwise; runs
-                                       as 6 when the planes do not fit) */
+                                       a source group), 16 K values per stage in a ring of 4 to 6: the B
+                                       operand is gathered and split once for twice the rows; equal to
+                                       9 to float32 rounding (default for 8 right-hand sides or more
+                                       otherwise; runs as 6 when the planes do not fit) */
 };
 
 /* vie_apply flags */

@@ -509,6 +509,7 @@ void build_apply_lists(Op& op) {
     upload(op.d_p2_ent, flat.empty() ? std::vector<int2>{make_int2(0, 0)} : flat);
     op.umma_ready = false;
     op.ws_ready = op.ws_packed = op.ws_pack_failed = false;
+    op.ws_tiles = 0;
     op.d_ws_r.release();
     op.d_ws_q.release();
 
@@ -733,6 +734,42 @@ void build_umma_lists(Op& op) {
     op.d_u1_pack.release();
     op.d_u2_pack.release();
     op.umma_ready = true;
+}
+
+// One or two row tiles per B tile (variants 9 and 10) for up to 32 columns.  Two read
+// and split the B operand once for twice the rows, which makes balanced lists 6 to 12%
+// faster, but halve the items: an SM's longest list may grow.  Both lists' loads, in
+// K stages, are known from the ranks; two tiles win up to 1.15 times the load of one
+// (35 arrays of 240 to 756 unknowns per atom, 8 to 32 columns: within 2% of the faster one;
+// us at 16 columns: 16 x 16 of 4^3 cubes 484 with one, 439 with two, 18 x 18 655 and 740,
+// lens-graded 9 x 9 159 and 223).  Atoms of one row tile leave the second one empty in phase 2:
+// always one (500 atoms of 108 unknowns: 733 against 813 us at 16 columns, 835 against 912 at 32).
+int ws_shape(const Op& op) {
+    if (op.ws_tiles) return op.ws_tiles;
+    const int nrt = (op.np + 127) / 128, per = (op.np + 7) / 8;
+    if (nrt == 1) return op.ws_tiles = 1;
+    std::map<std::tuple<int, int, int>, int64_t> groups;  // source box -> 8-row groups of the stacked R
+    std::vector<int64_t> chunks(op.N, 0);
+    for (const auto& b : op.blocks) {
+        const int G = (b.rank + 7) / 8;
+        if (G == 0) continue;
+        groups[{b.level, op.block_atoms[b.s_off], b.ns}] += G;
+        for (int s = 0; s < b.nt; ++s) chunks[op.block_atoms[b.t_off + s]] += G;
+    }
+    double load[2] = {0.0, 0.0};
+    for (int v = 0; v < 2; ++v) {
+        const int ks = v ? 16 : 32;
+        std::vector<double> w1, w2, loads;
+        std::vector<int> owner;
+        for (const auto& g : groups)
+            w1.insert(w1.end(), ((g.second + 15) / 16 + v) / (v + 1), tile_cost(8ll * per * std::get<2>(g.first), ks));
+        for (int64_t c : chunks) w2.insert(w2.end(), (nrt + v) / (v + 1), tile_cost(8 * c, ks));
+        for (const auto* w : {&w1, &w2}) {
+            lpt_assign(*w, op.ctx->n_sm, owner, loads);
+            load[v] += *std::max_element(loads.begin(), loads.end());
+        }
+    }
+    return op.ws_tiles = load[1] <= 1.15 * load[0] ? 2 : 1;
 }
 
 // Lists of the warp-specialised kernels (apply_ws.cu has the plane layouts).

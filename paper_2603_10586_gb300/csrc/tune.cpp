@@ -31,15 +31,10 @@ bool admissible(int precision, int v) {
 }
 
 int default_variant(const Op& op, int precision, int nrhs) {
-    // BF16x3: the warp-specialised kernel with one row tile per B tile while the B
-    // operand is narrow; wider, two row tiles per B tile, which gather and split
-    // it once for twice the factor rows
-    // (an atom of one row tile leaves the second one empty in phase 2: 733 against
-    // 813 us at 16 columns and 835 against 912 at 32 on 500 atoms of 108 unknowns; at 240
-    // unknowns two tiles win from the start, 1209 against 1217 us at 16 columns on the
-    // graded 24 x 24 array, 2510 against 2803 at 32 on the 32 x 32 array)
+    // BF16x3: the warp-specialised kernel, with two row tiles per B tile above 32
+    // columns, where gathering and splitting B weighs most, else as the lists balance
     if (precision == VIE_BF16X3 && nrhs >= 8)
-        return op.np <= 128 && nrhs <= 32 ? VIE_VAR_TCGEN05_WS_BF16X3 : VIE_VAR_TCGEN05_WS2_BF16X3;
+        return nrhs <= 32 && ws_shape(op) == 1 ? VIE_VAR_TCGEN05_WS_BF16X3 : VIE_VAR_TCGEN05_WS2_BF16X3;
     return nrhs == 1 ? (tile_pays(op, 1) ? VIE_VAR_SIMT_SHARED : VIE_VAR_SIMT_R1) : VIE_VAR_SIMT_R4;
 }
 
