@@ -172,24 +172,24 @@ __global__ void c64_to_c128(const float2* s, double2* d, int64_t n) {
 // B must not overlap Y.
 // ---------------------------------------------------------------------------
 constexpr int kGemmThr = 128;
-template <class T, int WN, int RA, int J>
+template <class T, int WN, int RA, int J, int K = RA == 2 ? 512 / (int)sizeof(T) : 16>
 struct GemmShape {
     static constexpr int WK = 4 / WN, TM = 16 * RA, TN = 2 * J * WN;
-    // (the narrow tile of small arrays takes its K range in few, longer stages: their
+    // (K: the narrow tile of small arrays takes its K range in few, longer stages: their
     // latency is all there is)
-    static constexpr int KC = RA == 2 ? 512 / (int)sizeof(T) : 16, KG = KC / WK;
+    static constexpr int KC = K, KG = KC / WK;
     static constexpr int LA = TM, LB = KC + kE<T>;  // A [K][row], B [column][K]
     static constexpr size_t a_pad = (size_t)KC * LA * sizeof(T);
     static constexpr size_t stage = a_pad + (size_t)TN * LB * sizeof(T);
 };
 
-template <class T, int WN, int RA, int J>
+template <class T, int WN, int RA, int J, int K>
 __global__ void __launch_bounds__(kGemmThr, 3) type_gemm(const T* __restrict__ M, int np, int tile_rows,
                                                          const int* __restrict__ atoms, int n_atoms, int nrhs,
                                                          const T* __restrict__ B, int64_t ldb, const T* ADD,
                                                          int64_t ldadd, T* Y, int64_t ldy,
                                                          const int2* __restrict__ colr, int prob) {
-    using S = GemmShape<T, WN, RA, J>;
+    using S = GemmShape<T, WN, RA, J, K>;
     constexpr int E = kE<T>, UR = S::TM / E, UK = S::KC / E;   // 16-byte units per K value of A, per column of B
     constexpr int KA = kGemmThr / UR, CB = kGemmThr / UK;      // K values of A, columns of B staged at a time
     constexpr int NB = (S::TN + CB - 1) / CB;
@@ -374,13 +374,13 @@ void conj_transpose_blocks(const void* src, void* dst, int T, int np, bool c128,
 }
 
 namespace {
-template <class T, int WN, int RA, int J>
+template <class T, int WN, int RA, int J, int K = GemmShape<T, WN, RA, J>::KC>
 void launch_gemm(const T* M, int np, const int* atoms, int na, int nrhs, const T* B, int64_t ldb, const T* ADD,
                  int64_t ldadd, T* Y, int64_t ldy, const int2* colr, int prob, cudaStream_t s) {
-    using S = GemmShape<T, WN, RA, J>;
+    using S = GemmShape<T, WN, RA, J, K>;
     const int nt = (np + S::TM - 1) / S::TM, tile_rows = ((np + nt - 1) / nt + 1) / 2 * 2;  // equal, even pieces
     const dim3 grid((np + tile_rows - 1) / tile_rows, (unsigned)(((int64_t)na * nrhs + S::TN - 1) / S::TN));
-    type_gemm<T, WN, RA, J><<<grid, kGemmThr, 0, s>>>(M, np, tile_rows, atoms, na, nrhs, B, ldb, ADD, ldadd, Y, ldy,
+    type_gemm<T, WN, RA, J, K><<<grid, kGemmThr, 0, s>>>(M, np, tile_rows, atoms, na, nrhs, B, ldb, ADD, ldadd, Y, ldy,
                                                       colr, prob);
     VIE_CHECK_LAUNCH();
 }
@@ -405,12 +405,16 @@ void self_gemm(Op& op, const TM* M, const TX* X, int64_t ldx, const TX* C, int64
         int64_t ldadd = mode == 0 ? ldc : ldx;
         const int prob = op.type_prob.empty() ? 0 : op.type_prob[t];
         // the widest tile that gives every SM two CTAs; the narrowest (32 rows, four
-        // warps along K) when none does
+        // warps along K) when none does.  Blocks of up to 32 rows (one voxel per edge) would
+        // leave most of a 64-row tile empty: 32 rows x 32 columns (complex128: 16), 16 K values
+        // per stage (6 unknowns, 576 atoms x 33 columns: 9.0 -> 6.1 us; complex128 131 -> 70 us).
         const int64_t rt = (np + 63) / 64, cols = (int64_t)na * nrhs, want = 2 * op.ctx->n_sm;
         auto enough = [&](int tn) { return rt * ((cols + tn - 1) / tn) >= want; };
 #define VIE_GEMM(WN, RA) \
     launch_gemm<TX, WN, RA, J>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s)
-        if (enough(8 * J)) VIE_GEMM(4, 4);
+        if (np <= 32)
+            launch_gemm<TX, J / 2, 2, 4, 16>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s);
+        else if (enough(8 * J)) VIE_GEMM(4, 4);
         else if (enough(4 * J)) VIE_GEMM(2, 4);
         else if (enough(2 * J)) VIE_GEMM(1, 4);
         else launch_gemm<TX, 1, 2, 4>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s);

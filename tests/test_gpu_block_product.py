@@ -1,0 +1,59 @@
+"""The self-block product (preconditioner) where its tiles lost time: blocks of one voxel per
+edge, which leave most of a 64-row tile empty."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+def _precond(g, nrhs, precision):
+    """(us per call on the device, worst column's error against the exported inverses)"""
+    import torch
+    from paper_2603_10586_gb300 import vie
+    ctx = vie.Context(0)
+    op = vie.Operator(ctx, g)
+    wide = precision == "C128"
+    x = workloads.random_complex(op.n, 6, nrhs).T.astype(np.complex128 if wide else np.complex64).copy()
+    X = torch.from_numpy(x).cuda()
+    Y = torch.empty_like(X)
+    call = lambda: op.precond(X.data_ptr(), Y.data_ptr(), nrhs, getattr(vie, precision))  # noqa: E731
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        for _ in range(20):
+            call()
+    times = []
+    for _ in range(6):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        graph.replay()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) * 50.0)
+    v = x.astype(complex).reshape(nrhs, g.n_atoms, op.np)
+    ref = np.zeros_like(v)
+    for t in range(len(g.sides)):
+        ref[:, g.types == t] = v[:, g.types == t] @ op.export_block(2, t).T
+    ref = ref.reshape(nrhs, -1)
+    err = (np.linalg.norm(Y.cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)).max()
+    op.close()
+    ctx.close()
+    return min(times), err
+
+
+# six products per sum: float32 rounding of a few terms, float64 likewise
+@pytest.mark.parametrize("ns,nrhs", [(1, 1), (3, 5), (11, 3), (24, 33)])
+@pytest.mark.parametrize("precision,tol", [("C64", 1e-6), ("C128", 1e-14)])
+def test_one_voxel_blocks(ns, nrhs, precision, tol):
+    assert _precond(workloads.graded_array(ns, 1, 2), nrhs, precision)[1] < tol
+
+
+def test_one_voxel_blocks_time():
+    # 24 x 24 atoms: 33 columns move 0.9 MB; one column is a launch (3.3 us).  64-row tiles: 2.5 times it
+    g = workloads.square_array(24, 1)
+    assert _precond(g, 33, "C64")[0] < 2.2 * _precond(g, 1, "C64")[0]
