@@ -404,19 +404,35 @@ void self_gemm(Op& op, const TM* M, const TX* X, int64_t ldx, const TX* C, int64
         const TX* ADD = mode == 0 ? C : (mode == 1 ? X : nullptr);
         int64_t ldadd = mode == 0 ? ldc : ldx;
         const int prob = op.type_prob.empty() ? 0 : op.type_prob[t];
-        // the widest tile that gives every SM two CTAs; the narrowest (32 rows, four
-        // warps along K) when none does.  Blocks of up to 32 rows (one voxel per edge) would
-        // leave most of a 64-row tile empty: 32 rows x 32 columns (complex128: 16), 16 K values
-        // per stage (6 unknowns, 576 atoms x 33 columns: 9.0 -> 6.1 us; complex128 131 -> 70 us).
+        // The widest tile that gives every SM two CTAs; the narrowest (32 rows, four
+        // warps along K) when none does.  complex128 keeps its SM's float64 units busy whatever
+        // the width, so there the SM with the most columns decides, and of the widths with
+        // two CTAs per SM the one with the fewest such columns is taken (a narrower one from 2%
+        // on; us: 81 atoms of 240 unknowns x 33 columns 1443 -> 1091, 256 x 16 1920 -> 1681,
+        // 49 of 450 x 64 5539 -> 4850; complex float32 loses nothing by its widest tiles).  Blocks
+        // of up to 32 rows (one voxel per edge) would leave most of a 64-row tile empty: 32
+        // rows x 32 columns (complex128: 16), 16 K values per stage (6 unknowns, 576 atoms x 33
+        // columns: 9.0 -> 6.1 us; complex128 131 -> 70 us).
         const int64_t rt = (np + 63) / 64, cols = (int64_t)na * nrhs, want = 2 * op.ctx->n_sm;
-        auto enough = [&](int tn) { return rt * ((cols + tn - 1) / tn) >= want; };
+        int width = 3;  // 8 J, 4 J or 2 J columns, or the narrowest
+        double least = 0.0;
+        for (int w = 0; w < 3; ++w) {
+            const int tn = 8 * J >> w;
+            const int64_t ctas = rt * ((cols + tn - 1) / tn);
+            if (ctas < want) continue;
+            const double most = sizeof(TX) == 16 ? (ctas + op.ctx->n_sm - 1) / op.ctx->n_sm * tn * (1.0 + 0.02 * w) : 1.0;
+            if (width == 3 || most < least) {
+                width = w;
+                least = most;
+            }
+        }
 #define VIE_GEMM(WN, RA) \
     launch_gemm<TX, WN, RA, J>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s)
         if (np <= 32)
             launch_gemm<TX, J / 2, 2, 4, 16>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s);
-        else if (enough(8 * J)) VIE_GEMM(4, 4);
-        else if (enough(4 * J)) VIE_GEMM(2, 4);
-        else if (enough(2 * J)) VIE_GEMM(1, 4);
+        else if (width == 0) VIE_GEMM(4, 4);
+        else if (width == 1) VIE_GEMM(2, 4);
+        else if (width == 2) VIE_GEMM(1, 4);
         else launch_gemm<TX, 1, 2, 4>(Mt, np, atoms, na, nrhs, Bop, ldb, ADD, ldadd, Y, ldy, op.colr, prob, s);
 #undef VIE_GEMM
     }

@@ -1,5 +1,6 @@
 """The self-block product (preconditioner) where its tiles lost time: blocks of one voxel per
-edge, which leave most of a 64-row tile empty."""
+edge, which leave most of a 64-row tile empty, and complex128 columns that left most SMs
+waiting for the last of their tiles."""
 import numpy as np
 import pytest
 
@@ -57,3 +58,15 @@ def test_one_voxel_blocks_time():
     # 24 x 24 atoms: 33 columns move 0.9 MB; one column is a launch (3.3 us).  64-row tiles: 2.5 times it
     g = workloads.square_array(24, 1)
     assert _precond(g, 33, "C64")[0] < 2.2 * _precond(g, 1, "C64")[0]
+
+
+@pytest.mark.parametrize("ns,nv,nrhs", [(9, 4, 33), (9, 4, 24), (7, 5, 64), (16, 4, 16), (8, 3, 33)])
+def test_float64_columns(ns, nv, nrhs):
+    # sums of up to 450 products in float64
+    assert _precond(workloads.square_array(ns, nv), nrhs, "C128")[1] < 1e-13
+
+
+def test_float64_columns_time():
+    # 33 columns of 81 atoms of 240 unknowns as 336 tiles: three on some SMs, 2.2 on average
+    g = workloads.square_array(9, 4)
+    assert _precond(g, 33, "C128")[0] / 33 < 1.03 * _precond(g, 24, "C128")[0] / 24
