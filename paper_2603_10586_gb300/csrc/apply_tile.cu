@@ -467,8 +467,11 @@ int tile_pass_cols(int64_t part_total, int nrhs, size_t elem) {
 // shared factors (gold atoms on a spiral, 3^3 cubes, us): 2 columns pay, 400 atoms 1192 -> 922;
 // one column does not, 500 atoms 795 -> 1206, unless the per-block kernel, a CTA for 128 rows
 // of an atom, has too few CTAs to hide its loads: 60 atoms 218 -> 108, 150 339 -> 281,
-// 200 395 -> 392, 300 523 -> 651.  (complex128 padding costs more: 3 columns.)
+// 200 395 -> 392, 300 523 -> 651.  (complex128 padding costs more: 3 columns.)  Nor do
+// the four launches pay for up to four atoms x four columns, or five atoms x one, where the
+// per-block kernels' two have a chain of a few blocks (2 atoms 20.0 -> 10.1 us, 5 20.8 -> 18.1).
 bool tile_pays(const Op& op, int nrhs) {
+    if (op.fprec != VIE_C128 && (op.N <= 4 ? nrhs <= 4 : op.N == 5 && nrhs == 1)) return false;
     const double least = op.fprec == VIE_C128 || nrhs == 1 ? 3.0 : 2.0;
     const bool few = op.fprec != VIE_C128 && 2 * op.n_p2_items < 3 * op.ctx->n_sm;
     return op.share_mean * nrhs >= least || few;
