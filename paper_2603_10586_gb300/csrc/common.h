@@ -250,7 +250,7 @@ struct Op {
     // tile), phase 1 runs and t places of the stacked 8-row groups, phase 2 chunks
     // per atom
     bool ws_ready = false, ws_packed = false, ws_pack_failed = false;
-    mutable int ws_tiles = 0;  // row tiles per B tile that up to 32 columns take (ws_shape; 0: not known yet)
+    int ws_tiles = 1;  // row tiles per B tile that up to 32 columns take (build_ws_lists)
     int ws_ncls = 0, n_ws1[2] = {0, 0};
     int64_t ws_r_units = 0, ws_q_chunks = 0, ws_t_total = 0;
     DevBuf d_ws_cls, d_ws_r, d_ws_q, d_ws_grp, d_ws_kptr, d_ws_qidx, d_ws_tidx;
@@ -478,7 +478,7 @@ void apply_far_simt32(Op& op, const float2* x, int64_t ldx, float2* F, int64_t l
                       cudaStream_t s);
 // far apply of float32 vectors by the variant chosen for (precision, nrhs)
 void far32(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, int nrhs, int precision, cudaStream_t s);
-int far_variant(const Op& op, int precision, int nrhs);
+int far_variant(Op& op, int precision, int nrhs);
 // time the admissible variants for (precision, nrhs), keep the fastest
 int tune_far(Op& op, int precision, int nrhs, cudaStream_t s, std::vector<int>& cand, std::vector<double>& ms);
 int tune_entry(Op& op, int precision, int nrhs, int force, vie_tune_result* res, cudaStream_t s);
@@ -498,7 +498,6 @@ void apply_far_umma_packed(Op& op, const float2* x, int64_t ldx, float2* F, int6
 // warp-specialised variants: lists (host.cpp), planes (false when the free memory
 // cannot hold them; the unpacked kernel runs instead), scratch for nrhs columns
 void build_ws_lists(Op& op);
-int ws_shape(const Op& op);  // 1 or 2 row tiles per B tile for up to 32 columns
 bool ws_pack(Op& op, cudaStream_t s);
 void ws_reserve(Op& op, int nrhs);
 size_t ws_plane_bytes(const Op& op);

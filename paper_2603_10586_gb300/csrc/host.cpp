@@ -326,10 +326,11 @@ void lpt_assign(const std::vector<double>& w, int nproc, std::vector<int>& owner
 // ---------------------------------------------------------------------------
 static void pack_lpt(const std::vector<int4>& items, const std::vector<double>& w, int ncta,
                      std::vector<int4>& out_items, std::vector<int>& cta_ptr, std::vector<int>* perm = nullptr,
-                     const std::vector<uint64_t>* key = nullptr) {
+                     const std::vector<uint64_t>* key = nullptr, double* most = nullptr) {
     std::vector<int> owner;
     std::vector<double> loads;
     lpt_assign(w, ncta, owner, loads);
+    if (most) *most = *std::max_element(loads.begin(), loads.end());
     std::vector<std::vector<int>> per(ncta);
     // within a CTA keep the heaviest items first, or, given a spatial key, the
     // items in key order: every CTA then sweeps the array in the same
@@ -509,7 +510,6 @@ void build_apply_lists(Op& op) {
     upload(op.d_p2_ent, flat.empty() ? std::vector<int2>{make_int2(0, 0)} : flat);
     op.umma_ready = false;
     op.ws_ready = op.ws_packed = op.ws_pack_failed = false;
-    op.ws_tiles = 0;
     op.d_ws_r.release();
     op.d_ws_q.release();
 
@@ -736,42 +736,6 @@ void build_umma_lists(Op& op) {
     op.umma_ready = true;
 }
 
-// One or two row tiles per B tile (variants 9 and 10) for up to 32 columns.  Two read
-// and split the B operand once for twice the rows, which makes balanced lists 6 to 12%
-// faster, but halve the items: an SM's longest list may grow.  Both lists' loads, in
-// K stages, are known from the ranks; two tiles win up to 1.15 times the load of one
-// (35 arrays of 240 to 756 unknowns per atom, 8 to 32 columns: within 2% of the faster one;
-// us at 16 columns: 16 x 16 of 4^3 cubes 484 with one, 439 with two, 18 x 18 655 and 740,
-// lens-graded 9 x 9 159 and 223).  Atoms of one row tile leave the second one empty in phase 2:
-// always one (500 atoms of 108 unknowns: 733 against 813 us at 16 columns, 835 against 912 at 32).
-int ws_shape(const Op& op) {
-    if (op.ws_tiles) return op.ws_tiles;
-    const int nrt = (op.np + 127) / 128, per = (op.np + 7) / 8;
-    if (nrt == 1) return op.ws_tiles = 1;
-    std::map<std::tuple<int, int, int>, int64_t> groups;  // source box -> 8-row groups of the stacked R
-    std::vector<int64_t> chunks(op.N, 0);
-    for (const auto& b : op.blocks) {
-        const int G = (b.rank + 7) / 8;
-        if (G == 0) continue;
-        groups[{b.level, op.block_atoms[b.s_off], b.ns}] += G;
-        for (int s = 0; s < b.nt; ++s) chunks[op.block_atoms[b.t_off + s]] += G;
-    }
-    double load[2] = {0.0, 0.0};
-    for (int v = 0; v < 2; ++v) {
-        const int ks = v ? 16 : 32;
-        std::vector<double> w1, w2, loads;
-        std::vector<int> owner;
-        for (const auto& g : groups)
-            w1.insert(w1.end(), ((g.second + 15) / 16 + v) / (v + 1), tile_cost(8ll * per * std::get<2>(g.first), ks));
-        for (int64_t c : chunks) w2.insert(w2.end(), (nrt + v) / (v + 1), tile_cost(8 * c, ks));
-        for (const auto* w : {&w1, &w2}) {
-            lpt_assign(*w, op.ctx->n_sm, owner, loads);
-            load[v] += *std::max_element(loads.begin(), loads.end());
-        }
-    }
-    return op.ws_tiles = load[1] <= 1.15 * load[0] ? 2 : 1;
-}
-
 // Lists of the warp-specialised kernels (apply_ws.cu has the plane layouts).
 void build_ws_lists(Op& op) {
     if (op.ws_ready) return;
@@ -871,6 +835,7 @@ void build_ws_lists(Op& op) {
     upload(op.d_ws_qidx, qidx);
     upload(op.d_ws_tidx, tidx);
     // items per tile shape, mapped to one CTA per SM
+    double load[2];  // the longest lists of the two phases, in K stages
     for (int v = 0; v < 2; ++v) {
         const int ks = v ? 16 : 32;
         std::vector<WsItem1> i1;
@@ -898,21 +863,32 @@ void build_ws_lists(Op& op) {
                 k2.push_back(zc[a]);
             }
         auto place = [&](auto& items, const std::vector<double>& w, const std::vector<uint64_t>& key, DevBuf& d_items,
-                         DevBuf& d_cta) {
+                         DevBuf& d_cta) -> double {
             using I = typename std::decay_t<decltype(items)>::value_type;
             std::vector<int4> dummy(items.size(), make_int4(0, 0, 0, 0)), out;
             std::vector<int> cta, perm;
-            pack_lpt(dummy, w, n_cta, out, cta, &perm, &key);
+            double most = 0.0;
+            pack_lpt(dummy, w, n_cta, out, cta, &perm, &key, &most);
             std::vector<I> sorted(std::max<size_t>(1, items.size()));
             for (size_t i = 0; i < perm.size(); ++i) sorted[i] = items[perm[i]];
             upload(d_items, sorted);
             upload(d_cta, cta);
+            return most;
         };
         op.n_ws1[v] = (int)i1.size();
-        place(i1, w1, k1, op.d_ws1_items[v], op.d_ws1_cta[v]);
-        place(i2, w2, k2, op.d_ws2_items[v], op.d_ws2_cta[v]);
+        load[v] = place(i1, w1, k1, op.d_ws1_items[v], op.d_ws1_cta[v]) +
+                  place(i2, w2, k2, op.d_ws2_items[v], op.d_ws2_cta[v]);
         upload(op.d_ws_runs[v], runs.empty() ? std::vector<WsRun>{WsRun{}} : runs);
     }
+    // Which of them up to 32 columns take (variant 9 or 10).  Two row tiles per B tile read
+    // and split the B operand once for twice the rows, which makes balanced lists 6 to 12%
+    // faster, but halve the items: an SM's longest list may grow.  They win up to 1.15
+    // times the load (35 arrays of 240 to 756 unknowns per atom, 8 to 32 columns: within 2% of the
+    // faster one; us at 16 columns: 16 x 16 of 4^3 cubes 484 with one, 439 with two, 18 x 18 655 and
+    // 740, lens-graded 9 x 9 159 and 223).  Atoms of one row tile leave the second one empty in
+    // phase 2: always one (500 atoms of 108 unknowns: 733 against 813 us at 16 columns, 835 against
+    // 912 at 32).
+    op.ws_tiles = nrt > 1 && load[1] <= 1.15 * load[0] ? 2 : 1;
     op.ws_ready = true;
 }
 

@@ -30,11 +30,13 @@ bool admissible(int precision, int v) {
             v == VIE_VAR_TCGEN05_WS_BF16X3 || v == VIE_VAR_TCGEN05_WS2_BF16X3);
 }
 
-int default_variant(const Op& op, int precision, int nrhs) {
+int default_variant(Op& op, int precision, int nrhs) {
     // BF16x3: the warp-specialised kernel, with two row tiles per B tile above 32
-    // columns, where gathering and splitting B weighs most, else as the lists balance
-    if (precision == VIE_BF16X3 && nrhs >= 8)
-        return nrhs <= 32 && ws_shape(op) == 1 ? VIE_VAR_TCGEN05_WS_BF16X3 : VIE_VAR_TCGEN05_WS2_BF16X3;
+    // columns, where gathering and splitting B weighs most, else as its lists balance
+    if (precision == VIE_BF16X3 && nrhs >= 8) {
+        if (nrhs <= 32) build_ws_lists(op);
+        return nrhs <= 32 && op.ws_tiles == 1 ? VIE_VAR_TCGEN05_WS_BF16X3 : VIE_VAR_TCGEN05_WS2_BF16X3;
+    }
     return nrhs == 1 ? (tile_pays(op, 1) ? VIE_VAR_SIMT_SHARED : VIE_VAR_SIMT_R1) : VIE_VAR_SIMT_R4;
 }
 
@@ -51,7 +53,7 @@ void far_grouped(Op& op, const float2* x, int64_t ldx, float2* F, int64_t ldf, i
 
 }  // namespace
 
-int far_variant(const Op& op, int precision, int nrhs) {
+int far_variant(Op& op, int precision, int nrhs) {
     auto it = op.variant.find({precision, bucket(nrhs)});
     return it != op.variant.end() ? it->second : default_variant(op, precision, nrhs);
 }
