@@ -72,10 +72,13 @@ enum vie_precision {
 /* Implementations of the far part of a complex float32 apply (the paper's
  * method fixes what is computed, not how; these are the kernel variants the
  * autotuner chooses between).  The SIMT variants read every factor element
- * once per group of 1, or of at least 2, 4 or 8 right-hand sides (when translated
- * copies or right-hand sides give a factor three or more columns, all of them run
- * the register tiles, which take up to 64 columns of a factor together); the
- * tensor-core variants compute in split bf16 (admissible for VIE_BF16X3 only). */
+ * once per group of 1, or of at least 2, 4 or 8 right-hand sides: by per-block
+ * kernels, or, for 2, 4 and 8, by the register tiles, which take up to 64 columns
+ * (translated copies x right-hand sides) of a factor together.  The tiles run where a
+ * factor has two columns or more on average, on one column three, and on operators of
+ * fewer than ~230 128-row pieces of atoms; not for the smallest products (four atoms x four
+ * columns, five x one).  vie_tune measures both forms.  The tensor-core variants compute in
+ * split bf16 (admissible for VIE_BF16X3 only). */
 enum vie_variant {
     VIE_VAR_AUTO = 0,
     VIE_VAR_SIMT_R1 = 1,
@@ -91,7 +94,7 @@ enum vie_variant {
                                their factors (translated copies) are applied together, each factor
                                element read once per group of up to 64 copies; partial products are
                                summed per target atom in a fixed order (default for one right-hand
-                               side when the operator has translated copies) */,
+                               side where the register tiles run, see above) */,
     VIE_VAR_TCGEN05_WS_BF16X3 = 9 /* the factors split once into bf16 planes, held once per factor
                                      storage (translated copies share them), in a warp-specialised
                                      persistent kernel (one CTA per SM): a warp moves the A planes by

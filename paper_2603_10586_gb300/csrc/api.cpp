@@ -108,7 +108,8 @@ void op_reserve(Op& op, int nrhs, int precision, cudaStream_t s) {
     if (op.d_t.bytes < need) op.d_t.alloc(need);
     const size_t need_x = (size_t)op.n() * nrhs * sizeof(float4);
     if (op.fprec == VIE_C64 && op.d_xs.bytes < need_x) op.d_xs.alloc(need_x);
-    if (tile_pays(op, nrhs)) tile_reserve(op, nrhs, sizeof(double2), s);  // float64-accurate residual, all-float64 applies
+    // float64-accurate residual, all-float64 applies
+    if (tile_pays(op, nrhs)) tile_reserve(op, nrhs, sizeof(double2), s);
     if (op.fprec == VIE_C64) {  // the inner products that run register tiles
         const int inner = precision == VIE_BF16X3 ? VIE_BF16X3 : VIE_C64;
         int cols = 0;

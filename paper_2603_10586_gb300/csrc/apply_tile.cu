@@ -29,11 +29,11 @@
 // Measured on one GB300 (fused apply, against the kernels that read a factor once
 // per four copies of one right-hand side or once per four right-hand sides):
 //   4 x 4 array of 3^3 cubes, 1 column, complex float32       38 -> 32 us
-//   16 x 16 array of 6^3 cubes, 1 column, complex float32    953 -> 533 us
+//   16 x 16 array of 6^3 cubes, 1 column, complex float32    953 -> 486 us
 //   28 x 28 array of 3^3 cubes, 5 columns, complex float32  4105 -> 1132 us
-//   16 x 16 array of 4^3 cubes, 24 columns, double-float    20.9 -> 17.3 ms
-//   12 x 12 array of 3^3 cubes, 3 columns, complex float64  3840 -> 2102 us
-//    8 x 8 array of 3^3 cubes, 1 column, complex float64     642 -> 447 us
+//   16 x 16 array of 4^3 cubes, 24 columns, double-float    20.9 -> 17.0 ms
+//   12 x 12 array of 3^3 cubes, 3 columns, complex float64  3840 -> 2079 us
+//    8 x 8 array of 3^3 cubes, 1 column, complex float64     642 -> 400 us
 #include <algorithm>
 #include <atomic>
 
@@ -360,9 +360,8 @@ __device__ __forceinline__ void tile_rows(unsigned char* smem, const TileArgs& a
 
 // blockIdx.x: item; its column tiles are dealt out along blockIdx.y
 template <class TF, class TX, int PHASE>
-__global__ void __launch_bounds__(kThr, std::is_same<TX, float4>::value ? 4 : 3) k_tile(TileArgs a, const TF* __restrict__ fac,
-                                                                        const TX* __restrict__ in,
-                                                                        TX* __restrict__ out) {
+__global__ void __launch_bounds__(kThr, std::is_same<TX, float4>::value ? 4 : 3)
+k_tile(TileArgs a, const TF* __restrict__ fac, const TX* __restrict__ in, TX* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char tile_smem[];
     constexpr int J = kJ<TX>, H = J / 2;  // columns per thread: full, and for the last few
     const FarTile it = a.items[blockIdx.x];
@@ -568,7 +567,8 @@ void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nr
             VIE_CHECK_LAUNCH();
         }
         k_tile_sum<TX, TO><<<dim3(op.n_p2_items, nc), 128, 0, s>>>(
-            op.d_p2_items.as<int4>(), op.d_p2_csr.as<int>(), op.d_pbase.as<long long>(), P, op.part_total, op.np, F, ldf, c0, op.colr);
+            op.d_p2_items.as<int4>(), op.d_p2_csr.as<int>(), op.d_pbase.as<long long>(), P, op.part_total, op.np, F, ldf,
+            c0, op.colr);
         VIE_CHECK_LAUNCH();
     }
 }

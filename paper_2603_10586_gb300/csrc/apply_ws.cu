@@ -25,15 +25,15 @@
 // One persistent CTA per SM; the roles run concurrently and meet on mbarriers
 // instead of CTA-wide barriers:
 //   warp 4     starts the bulk copies of the A planes of every K stage (32 KiB)
-//              into the next free slot of a ring of 3 to 6 stages (as many as fit
+//              into the next free slot of a ring of 4 to 6 stages (as many as fit
 //              beside the B planes of the widest tile), a lane per copy;
-//   warps 5-12 up to four groups of two warps (no more than the ring has
+//   warps 5-12 four groups of two warps (never more than the ring has
 //              stages) load, split and store the B operand (x gathered over
 //              the source atoms, or t) of a stage; group q takes the stages
-//              g = q mod G and gathers a stage's values into registers before
-//              it waits for the stage's slot, so the loads of G stages are in
+//              g = q mod 4 and gathers a stage's values into registers before
+//              it waits for the stage's slot, so the loads of four stages are in
 //              flight while the MMAs run;
-//   warp 13    one thread issues the 8 MMAs of a stage once its A copies have
+//   warp 13    one elected lane issues the 8 MMAs of a stage once its A copies have
 //              landed and its B planes are stored, and commits them to the
 //              slot's "empty" barrier (the producers refill it) and, at the end
 //              of a tile, to the tile's accumulator barrier;
@@ -185,8 +185,8 @@ constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }  //
 // the four wide MMAs of one K step (16): A unit and B stacks at the given low
 // words (without LBO), accumulator at tm
 template <int PHASE>
-__device__ __forceinline__ void mma_kstep_ws(uint32_t a, uint32_t b0, uint32_t b1, uint32_t tm, uint32_t id4, uint32_t id2,
-                                             uint32_t acc0) {
+__device__ __forceinline__ void mma_kstep_ws(uint32_t a, uint32_t b0, uint32_t b1, uint32_t tm, uint32_t id4,
+                                             uint32_t id2, uint32_t acc0) {
     using P = APlanes<PHASE>;
     constexpr uint32_t ah = desc_hi(P::sbo), bh = desc_hi(128), l = (P::lbo >> 4) << 16, p = P::plane >> 4;
     // planes: 0 re hi, 1 re lo, 2 im hi, 3 im lo
@@ -470,7 +470,7 @@ __device__ void ws_teardown(WsCtl& ctl, uint32_t ns, int* err) {
         for (uint32_t g = ctl.g_mma; g < ctl.g_tma; ++g)
             mbar_wait_lim(smem_u32(&ctl.full_a[g % ns]), (g / ns) & 1, kWaitCycles);
     }
-    if (threadIdx.x == kWsWarpMma * 32 && ctl.g_mma > 0) {  // the thread that issued the MMAs
+    if (threadIdx.x == kWsWarpMma * 32 && ctl.g_mma > 0) {  // the last issued stage's commit
         const uint32_t g = ctl.g_mma - 1;
         mbar_wait_lim(smem_u32(&ctl.empty[g % ns]), (g / ns) & 1, kWaitCycles);
     }
@@ -674,7 +674,8 @@ __device__ void ws_run(WsCtl& ctl, const WsRing& ring, int nmax, long long lim, 
                     if (mine) {
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
-                            if (cb + i < ncol) o[(int64_t)(cb + i) * (PHASE == 1 ? 8 : ldo)] = make_float2(ra[i] + rb[i], ia[i] + ib[i]);
+                            if (cb + i < ncol)
+                                o[(int64_t)(cb + i) * (PHASE == 1 ? 8 : ldo)] = make_float2(ra[i] + rb[i], ia[i] + ib[i]);
                     }
                 }
             }
@@ -699,11 +700,13 @@ __device__ __forceinline__ void ws_body(const Args& a, float2* out, int64_t ldo,
     ws_teardown(ctl, ring.ns, err);
 }
 template <int MT>
-__global__ void __launch_bounds__(kWsThr, 1) u1w_kernel(WsArgs1 a, float2* t, int64_t ldt, int nmax, int* err, long long lim) {
+__global__ void __launch_bounds__(kWsThr, 1) u1w_kernel(WsArgs1 a, float2* t, int64_t ldt, int nmax, int* err,
+                                                         long long lim) {
     ws_body<MT, 1, WsTile1>(a, t, ldt, nmax, err, lim);
 }
 template <int MT>
-__global__ void __launch_bounds__(kWsThr, 1) u2w_kernel(WsArgs2 a, float2* F, int64_t ldf, int nmax, int* err, long long lim) {
+__global__ void __launch_bounds__(kWsThr, 1) u2w_kernel(WsArgs2 a, float2* F, int64_t ldf, int nmax, int* err,
+                                                         long long lim) {
     ws_body<MT, 2, WsTile2>(a, F, ldf, nmax, err, lim);
 }
 
@@ -759,8 +762,8 @@ __global__ void __launch_bounds__(256) k_x8(const float2* __restrict__ x, int64_
 }
 
 // Q: thread = one row of a chunk of 8 K values
-__global__ void __launch_bounds__(128) k_pack_q(const WsClass* __restrict__ cls, int ncls, int64_t total, int np, int nrt,
-                                                const float2* __restrict__ fac, unsigned char* __restrict__ planes) {
+__global__ void __launch_bounds__(128) k_pack_q(const WsClass* __restrict__ cls, int ncls, int64_t total, int np,
+                                                int nrt, const float2* __restrict__ fac, unsigned char* __restrict__ planes) {
     for (int64_t w = blockIdx.x; w < total * nrt; w += gridDim.x) {
         const int rt = (int)(w / total);
         const int64_t chunk = w - rt * total;
@@ -824,7 +827,8 @@ bool ws_pack(Op& op, cudaStream_t s) {
     if (op.ws_ncls > 0) {
         const int64_t w1 = op.ws_r_units * 16;
         k_pack_r<<<(unsigned)std::min<int64_t>((w1 + 255) / 256, 64ll * op.ctx->n_sm), 256, 0, s>>>(
-            op.d_ws_cls.as<WsClass>(), op.ws_ncls, w1, op.np, (op.np + 7) / 8, op.fac<float2>(), op.d_ws_r.as<unsigned char>());
+            op.d_ws_cls.as<WsClass>(), op.ws_ncls, w1, op.np, (op.np + 7) / 8, op.fac<float2>(),
+            op.d_ws_r.as<unsigned char>());
         VIE_CHECK_LAUNCH();
         k_pack_q<<<(unsigned)std::min<int64_t>(op.ws_q_chunks, 64ll * op.ctx->n_sm), 128, 0, s>>>(
             op.d_ws_cls.as<WsClass>(), op.ws_ncls, op.ws_q_chunks, op.np, (op.np + kM - 1) / kM, op.fac<float2>(),
@@ -862,7 +866,8 @@ static void apply_far_ws(Op& op, const float2* x, int64_t ldx, float2* F, int64_
         const int per = (op.np + 7) / 8;
         const int64_t chunks = (int64_t)op.N * per;
         for (int c0 = 0; c0 < nrhs; c0 += 65535) {
-            k_x8<<<dim3((unsigned)std::min<int64_t>((chunks + 255) / 256, 65535), (unsigned)std::min(nrhs - c0, 65535)), 256, 0, s>>>(
+            const dim3 grid((unsigned)std::min<int64_t>((chunks + 255) / 256, 65535), (unsigned)std::min(nrhs - c0, 65535));
+            k_x8<<<grid, 256, 0, s>>>(
                 x + c0 * ldx, ldx, op.np, per, chunks, nrhs, op.d_xs.as<float2>() + 8 * c0);
             VIE_CHECK_LAUNCH();
         }

@@ -111,8 +111,10 @@ void DevBuf::alloc(size_t b) {
         }
         if (cap > 0 && now > cap) {
             c->allocated.fetch_sub((int64_t)b);
-            throw Error{VIE_ERR_OOM, "allocation of " + std::to_string(b) + " bytes would exceed the context's cap of " +
-                                         std::to_string(cap) + " bytes", true};
+            throw Error{VIE_ERR_OOM,
+                        "allocation of " + std::to_string(b) + " bytes would exceed the context's cap of " +
+                            std::to_string(cap) + " bytes",
+                        true};
         }
     }
     // (the null stream names no stream to free on: such a buffer is not pooled)
@@ -548,7 +550,8 @@ void build_apply_lists(Op& op) {
             const auto& b = op.blocks[kv.second[0]];
             const int64_t cnt = (int64_t)kv.second.size();
             nmem += cnt;
-            n64 += (cnt + kTileMembers - 1) / kTileMembers * ((b.n + seg_len - 1) / seg_len) * ((b.rank + kTileRows1 - 1) / kTileRows1);
+            n64 += (cnt + kTileMembers - 1) / kTileMembers * ((b.n + seg_len - 1) / seg_len) *
+                   ((b.rank + kTileRows1 - 1) / kTileRows1);
         }
         op.share_mean = cls.empty() ? 1.0 : (double)nmem / (double)cls.size();
         const bool fine = op.share_mean >= 3.0 && n64 < 8 * (int64_t)op.ctx->n_sm;
@@ -573,7 +576,8 @@ void build_apply_lists(Op& op) {
             const auto& mem = kv.second;
             const auto& b = op.blocks[mem[0]];
             auto tiles = [](int rows, int most, auto&& f) {  // equal pieces of at most `most` rows
-                const int nt = (rows + most - 1) / most, per = ((rows + nt - 1) / nt + 1) / 2 * 2;  // even: 16-byte copies
+                const int nt = (rows + most - 1) / most;
+                const int per = ((rows + nt - 1) / nt + 1) / 2 * 2;  // even: 16-byte copies
                 for (int r0 = 0; r0 < rows; r0 += per) f(r0, std::min(per, rows - r0));
             };
             for (size_t g = 0; g < mem.size(); g += kTileMembers) {
@@ -858,7 +862,8 @@ void build_ws_lists(Op& op) {
         for (int a = 0; a < op.N; ++a)
             for (int rt = 0; rt < nrt; rt += v + 1) {
                 auto rows = [&](int t) { return std::max(0, std::min(128, op.np - t * 128)); };
-                i2.push_back(WsItem2{a, op.atom_prob.empty() ? 0 : op.atom_prob[a], rt, {rows(rt), v ? rows(rt + 1) : 0}});
+                const int prob = op.atom_prob.empty() ? 0 : op.atom_prob[a];
+                i2.push_back(WsItem2{a, prob, rt, {rows(rt), v ? rows(rt + 1) : 0}});
                 w2.push_back(tile_cost(8ll * (cnt[a + 1] - cnt[a]), ks));
                 k2.push_back(zc[a]);
             }

@@ -162,8 +162,8 @@ __global__ void c64_to_c128(const float2* s, double2* d, int64_t n) {
 // lives at a * np + r + c * ld.  A CTA of four warps takes 16 RA rows x 2 J WN
 // columns, the warps side by side and, where the columns are few, along K (WK =
 // 4 / WN groups added in order at the end); operands staged by cp.async through two
-// shared-memory buffers.  Bound by the float32 (float64) pipes; the launcher picks
-// the widest tile that still fills the GPU twice over.  (A 2 x 2 sub-tile per
+// shared-memory buffers.  Bound by the float32 (float64) pipes; self_gemm
+// picks the width.  (A 2 x 2 sub-tile per
 // thread and 32 x 32 per CTA, the kernel before, took 997 us for 61,440 columns of
 // np = 240 in float32, now 669 us, and 19 us for 16 columns of np = 108, now 9 us.)
 // ADD may be Y itself (y = Z_ii x + y in place): every output element is read
@@ -420,7 +420,8 @@ void self_gemm(Op& op, const TM* M, const TX* X, int64_t ldx, const TX* C, int64
             const int tn = 8 * J >> w;
             const int64_t ctas = rt * ((cols + tn - 1) / tn);
             if (ctas < want) continue;
-            const double most = sizeof(TX) == 16 ? (ctas + op.ctx->n_sm - 1) / op.ctx->n_sm * tn * (1.0 + 0.02 * w) : 1.0;
+            const int64_t per_sm = (ctas + op.ctx->n_sm - 1) / op.ctx->n_sm;
+            const double most = sizeof(TX) == 16 ? (double)(per_sm * tn) * (1.0 + 0.02 * w) : 1.0;
             if (width == 3 || most < least) {
                 width = w;
                 least = most;

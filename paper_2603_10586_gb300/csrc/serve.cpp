@@ -10,11 +10,12 @@
 //
 // The slot's context refuses allocations beyond the footprint its request
 // was admitted with (whole chunks that its pool of temporaries keeps count), so
-// an under-estimate cannot take memory that another request was promised: the allocation fails with VIE_ERR_OOM on the host,
-// and the request goes back to the head of the queue with twice the
-// footprint (at most the whole budget), to run again once that much is free.
-// With the whole budget a request that lacks only the register tiles' scratch runs
-// without it; one that fails even so is rejected.
+// an under-estimate cannot take memory that another request was promised: the
+// allocation fails with VIE_ERR_OOM on the host, and the request goes back to
+// the head of the queue with twice the footprint (at most the whole budget), to
+// run again once that much is free.  With the whole budget a request that
+// lacks only the register tiles' scratch runs without it; one that fails even
+// so is rejected.
 #include <chrono>
 #include <cmath>
 #include <cstdlib>
