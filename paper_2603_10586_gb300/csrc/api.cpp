@@ -142,7 +142,7 @@ int guarded(vie_ctx* ctx, F&& f) {
         try {
             f();
         } catch (const Error& e) {
-            if (!e.memory || !ctx || ctx->c.admitted || !tile_give_back(ctx->c)) throw;
+            if (!e.memory || !ctx || ctx->c.admitted || !give_back_scratch(ctx->c)) throw;
             f();
         }
         if (ctx) ctx->c.err.clear();
@@ -361,6 +361,7 @@ int vie_assemble(vie_ctx* ctx, const vie_geometry* g, double wavelength, vie_op*
                     o.blocks.size(), o.t_assemble);
     });
     if (st == VIE_OK) {
+        ctx->c.ops.push_back(&op->o);
         ctx->ops.fetch_add(1);
         *out = op.release();
     }

@@ -478,7 +478,7 @@ bool tile_pays(const Op& op, int nrhs) {
 
 Op::~Op() {
     if (!ctx) return;
-    auto& v = ctx->tile_ops;
+    auto& v = ctx->ops;
     v.erase(std::remove(v.begin(), v.end(), this), v.end());
 }
 
@@ -494,8 +494,6 @@ bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
         return true;
     }
     if (capturing || (op.tile_oom && np + nt >= op.tile_oom)) return false;
-    auto& v = op.ctx->tile_ops;
-    if (std::find(v.begin(), v.end(), &op) == v.end()) v.push_back(&op);
     try {
         if (np + nt > ((size_t)256 << 20) && !op.ctx->admitted) {  // leave 1 GiB to the solver, as ws_pack does
             size_t free_b = 0, total_b = 0;
@@ -518,9 +516,13 @@ bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
     return true;
 }
 
-bool tile_give_back(Ctx& c) {
+bool give_back_scratch(Ctx& c) {
     bool any = false;
-    for (Op* o : c.tile_ops) {
+    for (Op* o : c.ops) {
+        for (DevBuf* b : {&o->d_pw, &o->d_fpart, &o->d_fI, &o->d_fdirs, &o->d_fout}) {
+            any |= b->bytes > 0;
+            b->release();
+        }
         const size_t held = o->d_part.bytes + o->d_ct.bytes;
         if (o->tile_pinned || held == 0) continue;
         o->d_part.release();

@@ -149,6 +149,7 @@ Op* get_union(const std::vector<Op*>& ops) {
                                     [](const Ctx::Union& a, const Ctx::Union& b) { return a.used < b.used; });
         c.unions.erase(lru);
     }
+    c.ops.push_back(U.get());
     c.unions.push_back(Ctx::Union{std::move(key), std::move(gens), std::move(U), ++c.union_clock});
     return c.unions.back().U.get();
 }

@@ -274,7 +274,8 @@ struct Op {
     // plane waves and fields: incident directions and polarisations, plane-wave
     // tables (at most 32 MB, or one direction's), partial sums, currents, results,
     // and the quadrature sphere of the cross sections.  What a vie_fields call
-    // leaves above kFieldsKeep is given back when it returns.
+    // leaves above kFieldsKeep is given back when it returns, the rest when a call is
+    // short of memory (no work is in flight on them between calls).
     DevBuf d_inc, d_pw, d_fpart, d_fI, d_fdirs, d_fout, d_sphere;
     static constexpr size_t kFieldsKeep = (size_t)64 << 20;
     size_t t_cap = 0, F_cap = 0;
@@ -311,7 +312,7 @@ struct Ctx {
     // a server's slot whose request is run again with more when it meets the cap, so that its
     // result does not depend on the cap (at the whole budget it makes do without scratch)
     bool admitted = false;
-    std::vector<Op*> tile_ops;  // operators that hold register-tile scratch
+    std::vector<Op*> ops;  // the operators of this context, joined ones among them
     // joined operators of recent vie_solve_batch calls (block-diagonal unions of
     // their problems), reused while the same operators with the same factors
     // come again; declared last so that they are freed first
@@ -512,9 +513,10 @@ bool tile_pays(const Op& op, int nrhs);
 bool far_tiled(const Op& op, int precision, int nrhs);  // tile_pays, or the autotuner's choice
 int tile_pass_cols(int64_t part_total, int nrhs, size_t elem);  // right-hand sides per pass
 bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s);
-// gives back the scratch of the context's operators (not what a caller's graph holds), for a
-// call that is short of memory; false when there was none
-bool tile_give_back(Ctx& c);
+// gives back the scratch that the context's operators keep between calls (register tiles,
+// unless a caller's graph holds theirs; plane waves and fields), for a call that is short of
+// memory; false when there was none
+bool give_back_scratch(Ctx& c);
 template <class TF, class TX, class TO>
 void apply_far_tile(Op& op, const TX* x, int64_t ldx, TO* F, int64_t ldf, int nrhs, cudaStream_t s, int first = 0,
                     int count = -1);  // columns [first, first + count) of the call (-1: all)
