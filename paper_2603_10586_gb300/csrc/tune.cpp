@@ -102,10 +102,27 @@ int tune_far(Op& op, int precision, int nrhs, cudaStream_t s, std::vector<int>& 
     const int64_t n = op.n();
     DevBuf x((size_t)n * nrhs * sizeof(float2)), F((size_t)n * nrhs * sizeof(float2));
     VIE_CUDA(cudaMemsetAsync(x.p, 0, (size_t)n * nrhs * sizeof(float2), s));
+    // the planes of 9 and 10 first: those of 7, one set per block, are many times larger, and
+    // stay only if 7 is chosen (or was before)
+    struct PackGuard {
+        Op& o;
+        bool keep;
+        ~PackGuard() {
+            if (keep) return;
+            o.d_u1_pack.release();
+            o.d_u2_pack.release();
+            o.umma_packed = false;
+        }
+    } packed{op, op.umma_packed || precision != VIE_BF16X3};
     if (precision == VIE_BF16X3) {
-        umma_prepare(op, s);
-        umma_pack(op, s);
         ws_pack(op, s);
+        umma_prepare(op, s);
+        try {
+            umma_pack(op, s);
+        } catch (const Error& e) {  // no room beside the others: 7 is timed as 6
+            if (!e.memory) throw;
+            op.umma_pack_failed = true;
+        }
     }
     cudaEvent_t e0, e1;
     VIE_CUDA(cudaEventCreate(&e0));
@@ -166,6 +183,7 @@ int tune_far(Op& op, int precision, int nrhs, cudaStream_t s, std::vector<int>& 
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    packed.keep |= best == VIE_VAR_TCGEN05_PACKED_BF16X3;
     op.variant[key] = best;
     if (best >= VIE_VAR_SIMT_R2 && best <= VIE_VAR_SIMT_R8) op.tiled[key] = best_form;
     else op.tiled.erase(key);
