@@ -402,15 +402,29 @@ int atom_chunks(const Op& op, int64_t blocks, int min_atoms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>({want, (int64_t)(op.N / min_atoms), (int64_t)64}));
 }
 
-// directions of one pass: their tables stay within 32 MB (or one direction's)
-int table_cols(const Op& op, int W) {
+
+// room in b for `want` columns of `per` bytes, or for as many as there is memory for
+int fit(DevBuf& b, size_t per, int want) {
+    while (b.bytes < per * want) {
+        try {
+            b.alloc(per * want);
+        } catch (const Error& e) {
+            if (!e.memory || want == 1) throw;
+            want = (want + 1) / 2;
+        }
+    }
+    return want;
+}
+
+// directions of one pass: their tables (op.d_pw) stay within 32 MB (or one direction's)
+int table_cols(Op& op, int W) {
     const size_t per = ((size_t)op.T * op.np + op.N) * sizeof(double2);
-    return (int)std::max<size_t>(1, std::min<size_t>({(size_t)W, ((size_t)32 << 20) / per, (size_t)65535}));
+    const size_t most = std::min<size_t>({(size_t)W, ((size_t)32 << 20) / per, (size_t)65535});
+    return fit(op.d_pw, per, (int)std::max<size_t>(1, most));
 }
 
 double2* tables(Op& op, const double* vec, double sign, const double* pol, int W, double2** ph, cudaStream_t s) {
     const size_t nV = (size_t)op.T * W * op.np;
-    grow(op.d_pw, (nV + (size_t)W * op.N) * sizeof(double2));
     double2* V = op.d_pw.as<double2>();
     *ph = V + nV;
     k_pw_tables<<<dim3(W, op.T + (op.N + 255) / 256), 256, 0, s>>>(geo_of(op), vec, sign, op.k, pol, W, V, *ph);
@@ -447,15 +461,16 @@ void rhs_kernel_launch(Op& op, const double* d_khat, const double* d_pol, int nr
 // far-field amplitudes of nrhs currents in npts directions: d_out[(c npts + p) 3 + d]
 void far_field_launch(Op& op, const void* d_I, int nrhs, const double* d_dirs, int npts, void* d_out,
                       cudaStream_t s) {
-    const int wc = std::min(table_cols(op, npts), sum_cols(nrhs, npts)), groups = (nrhs + kRC - 1) / kRC;
+    const int groups = (nrhs + kRC - 1) / kRC;
+    int wc = table_cols(op, sum_cols(nrhs, npts));
+    int nz = atom_chunks(op, (int64_t)wc * groups, 4);
+    const int per = (op.N + nz - 1) / nz;
+    nz = (op.N + per - 1) / per;
+    wc = fit(op.d_fpart, (size_t)nz * nrhs * 3 * sizeof(double2), wc);
     for (int w0 = 0; w0 < npts; w0 += wc) {
         const int W = std::min(wc, npts - w0);
         double2* ph;
         const double2* V = tables(op, d_dirs + 3 * w0, 1.0, nullptr, W, &ph, s);
-        int nz = atom_chunks(op, (int64_t)W * groups, 4);
-        const int per = (op.N + nz - 1) / nz;
-        nz = (op.N + per - 1) / per;
-        grow(op.d_fpart, (size_t)nz * W * nrhs * 3 * sizeof(double2));
         k_radiate<<<dim3(W, nz, groups), 256, 0, s>>>(geo_of(op), V, ph, W, w0, (const double2*)d_I, nrhs, 0, per, nz,
                                                       op.d_fpart.as<double2>());
         VIE_CHECK_LAUNCH();
@@ -494,11 +509,12 @@ void sphere_sum_launch(const void* d_F, const double* d_wt, int npts, int nrhs, 
 }
 
 void near_field_launch(Op& op, const void* d_I, int nrhs, const double* d_pts, int npts, void* d_out, cudaStream_t s) {
-    const int pc = sum_cols(nrhs, npts), groups = (nrhs + kRC - 1) / kRC;
+    const int groups = (nrhs + kRC - 1) / kRC;
+    int pc = sum_cols(nrhs, npts);
     int nz = atom_chunks(op, (int64_t)pc * groups, 1);
     const int per = (op.N + nz - 1) / nz;
     nz = (op.N + per - 1) / per;
-    grow(op.d_fpart, (size_t)nz * pc * nrhs * 3 * sizeof(double2));
+    pc = fit(op.d_fpart, (size_t)nz * nrhs * 3 * sizeof(double2), pc);
     for (int64_t p0 = 0; p0 < npts; p0 += pc) {
         const int P = (int)std::min<int64_t>(pc, npts - p0);
         k_near<<<dim3(P, nz, groups), 256, 0, s>>>(op.dmesh, geo_of(op), op.k, (const double2*)d_I, nrhs,

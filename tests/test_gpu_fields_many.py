@@ -27,3 +27,24 @@ def test_output_is_held_once(mode, nrhs, npts, budget):
         assert np.abs(out[:, at:at + 80] - want).max() <= 1e-13 * np.abs(want).max()
     op.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("budget", [22, 26])
+def test_passes_fit_a_small_budget(budget):
+    # 18 MB of amplitudes in a context of 22 and 26 MB: shorter passes, not VIE_ERR_OOM
+    from paper_2603_10586_gb300 import vie
+    rng = np.random.default_rng(3)
+    p = rng.uniform(0.5, 2.0, (6000, 3)) + [0, 0, 3.0]
+    d = p / np.linalg.norm(p, axis=1, keepdims=True)
+    out = []
+    for mb in (0, budget):
+        ctx = vie.Context(0, hbm_budget=mb << 20)
+        op = vie.Operator(ctx, workloads.vogel_gold(40, 2))
+        I = workloads.random_complex(op.n, 4, 64)
+        kh, pol = workloads.random_directions(64, 2)
+        out.append((op.far_field(I, d), op.near_field(I, p), op.sigma(I, kh, pol)))
+        op.close()
+        ctx.close()
+    for a, b in zip(*out):
+        # float64 sums of ~1,400 terms in another order
+        assert np.abs(a - b).max() <= 1e-11 * np.abs(a).max()
