@@ -517,6 +517,7 @@ bool tile_reserve(Op& op, int nrhs, size_t elem, cudaStream_t s) {
 }
 
 bool give_back_scratch(Ctx& c) {
+    cudaStreamSynchronize(c.stream);  // (what the failed call had started)
     bool any = false;
     for (Op* o : c.ops) {
         for (DevBuf* b : {&o->d_pw, &o->d_fpart, &o->d_fI, &o->d_fdirs, &o->d_fout}) {

@@ -38,3 +38,23 @@ def test_launches(atoms, nrhs, blocks, nv):
     assert (np.linalg.norm(Y.cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)).max() < 1e-5
     op.close()
     ctx.close()
+
+
+def test_grouped_kernels_keep_a_columns_order():
+    # the per-block kernels of 2, 4 and 8 right-hand sides sum every column alike
+    import torch
+    from paper_2603_10586_gb300 import vie
+    ctx = vie.Context(0)
+    op = vie.Operator(ctx, workloads.vogel_gold(4, 3))
+    op.compress(1e-5, vie.C64)
+    X = torch.from_numpy(workloads.random_complex(op.n, 5, 4).T.astype(np.complex64).copy()).cuda()
+    out = []
+    for v in (vie.VAR_SIMT_R2, vie.VAR_SIMT_R4, vie.VAR_SIMT_R8):
+        op.tune(vie.C64, 4, force=v)
+        Y = torch.zeros_like(X)
+        op.apply(X.data_ptr(), Y.data_ptr(), 4, vie.C64, vie.FUSE_PRECOND)
+        torch.cuda.synchronize()
+        out.append(Y.cpu().numpy())
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[1], out[2])
+    op.close()
+    ctx.close()
